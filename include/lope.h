@@ -211,13 +211,25 @@ lope_status lope_apply_host(const lope_grid* grid, const lope_stencil* stencil,
  *              builtin: 64 x 32 / 32 x 32) whose planes producer warps copy in;
  *              box functions and multi-stage steps: 64 x 16 tiles; BF16:
  *              64 x 4 tiles.
+ *            5 register strips (2D, FP32 / BF16 storage): each warp marches a
+ *              128-column strip along y with every fused sweep's rows in
+ *              registers.  Any function of any row pitch, except that BF16
+ *              storage, multi-stage steps (builtins and weight tables) and
+ *              run-time compiled functions (star functions, plain sweeps) need a
+ *              row length that is a multiple of 4.  tsteps is 8 (one field,
+ *              radius-1 star), 6 (three-field star) or 4, or less: 4, 2, 1;
+ *              a sweep count that is no multiple ends with launches of 4, 2
+ *              and 1 sweeps.  Multi-stage steps run one step per launch.
+ *              The planner's choice for calls of 12 or more sweeps; shorter
+ *              calls take the paths below.
  *            For grids whose row pitch is not a multiple of 16 bytes the
  *            planner takes trapezoid tiles fusing 4 sweeps in 2D (128 x 32
  *            for one field, 64 x 16 for several) and the plane march in 3D.
  *   tile_x, tile_y: tile shape for path 2 (tile_x in {32,64,128}, tile_y in
  *            {8,16,32}); for path 1, tile_y = 1 or 2 forces the short or the
  *            tall tiles (0: tall from 2^22 points in 2D, 2^26 in 3D).
- *   tsteps:  temporal depth k (sweeps fused per launch; path 2 only, 1..8).
+ *   tsteps:  temporal depth k (sweeps fused per launch): path 2 1..8, path 1 1 or
+ *            2, path 5 as above.
  *   graph:   0 auto, 1 capture the launch sequence in a CUDA graph, -1 never. */
 typedef struct {
   int path;

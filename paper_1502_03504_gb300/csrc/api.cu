@@ -209,12 +209,40 @@ bool choice_supported(StepArgs a, const Choice& c) {
     case kPathTrap: ok = trap2d_supported(a); break;
     case kPathDirect: ok = direct_supported(a); break;
     case kPathMarch: ok = march_supported(a); break;
+    case kPathStrip: ok = strip_supported(a); break;
     default: ok = false;
   }
   return ok && !(a.s.stages >= 2 && c.path != kPathTrap && c.k != 1);
 }
 
-Choice default_choice(const Geom& g, const StencilDesc& s, int* err) {
+// Sweeps of the next launch: the trapezoid takes any count up to its depth; the
+// strips run at their depth, then at 4, 2 and 1.
+int64_t next_depth(const Choice& c, int64_t left) {
+  if (c.path == kPathStrip) return strip_next_depth(c.k, left);
+  return std::min<int64_t>(c.k, left);
+}
+int64_t count_passes(const Choice& c, int64_t nsteps) {
+  int64_t n = nsteps / c.k;
+  for (int64_t left = nsteps - n * c.k; left > 0; left -= next_depth(c, left)) ++n;
+  return n;
+}
+
+// The register strips serve calls of at least kStripSteps sweeps (or steps).
+// Shorter calls keep the plans documented for them (see lope.h): callers that
+// query or log the plan of a short call see the path they always saw.
+constexpr int64_t kStripSteps = 12;
+
+// The strip choice for a grid, if the strips take it (they measured faster than
+// every other path there).
+bool strip_choice(StepArgs a, Choice* c) {
+  a.ksteps = a.s.stages >= 2 ? 1 : strip_kmax_of(a);
+  if (!strip_supported(a)) return false;
+  *c = {kPathStrip, 0, 0, a.ksteps};
+  return true;
+}
+
+Choice default_choice(const Geom& g, const StencilDesc& s, const void* const* in, int64_t nsteps,
+                      int* err) {
   StepArgs a = base_args(g, s, err, nullptr);
   for (int f = 0; f < g.nf; ++f) a.in[f] = reinterpret_cast<const void*>(uintptr_t(256));
   {
@@ -223,6 +251,21 @@ Choice default_choice(const Geom& g, const StencilDesc& s, int* err) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(tune_key(g, s));
     if (it != g_tune.end() && choice_supported(a, it->second)) return it->second;
+  }
+  if (nsteps >= kStripSteps) {
+    // Register strips, FP32 / BF16.  Measured on GB300 against the choices
+    // below (which the same calls took before): jacobi5 FP32 7094^2 x20
+    // (unaligned rows) 1.65 -> 0.38 ms, 100 x 200 x20 51 -> 39 us; star9r2 FP32
+    // 8192^2 x50 3.03 -> 1.72 ms; linear shallow water 4096^2 x3 x200 FP32 7.86
+    // -> 2.60 ms, BF16 7.17 -> 2.45; RK3 nonlinear shallow water FP32 4096^2 x50
+    // steps 14.2 -> 5.15 ms; a run-time compiled Gray-Scott FP32 4096^2 x100
+    // 3.99 -> 1.46 ms.  FP64 is bound by its arithmetic and stays below (256^2
+    // x100: 0.41 ms in trapezoid tiles, 0.46 in strips).
+    StepArgs b = a;
+    if (in)
+      for (int f = 0; f < g.nf; ++f) b.in[f] = in[f];
+    Choice c;
+    if (strip_choice(b, &c)) return c;
   }
   if (s.stages >= 2 && g.ndim == 2 && g.nf == 1 && g.dtype == kF32) {
     // Multi-stage steps of a single FP32 field: the fused trapezoid keeps the
@@ -294,8 +337,10 @@ Choice default_choice(const Geom& g, const StencilDesc& s, int* err) {
 }
 
 lope_status resolve(const Geom& g, const StencilDesc& s, const void* const* in,
-                    const lope_launch* cfg, int* err, Choice* c) {
-  Choice d = default_choice(g, s, err);
+                    int64_t nsteps, const lope_launch* cfg, int* err, Choice* c) {
+  // a caller's tile or depth without a path applies to the paths that have one
+  const bool shaped = cfg && (cfg->tsteps > 0 || cfg->tile_x > 0 || cfg->tile_y > 0);
+  Choice d = default_choice(g, s, in, shaped ? 0 : nsteps, err);
   if (cfg && cfg->path != kPathAuto) {
     d.path = cfg->path;
     d.tile_x = cfg->tile_x;
@@ -341,7 +386,7 @@ void log_plan(const Geom& g, const StencilDesc& s, const Choice& c, int64_t nste
   static const char* kinds[] = {"linear", "jacobi5", "diff7", "star9r2", "swe_cgrid", "swe_flux",
                                 "source"};
   static const char* dtypes[] = {"f64", "f32", "bf16"};
-  static const char* paths[] = {"auto", "tma", "trapezoid", "direct", "march"};
+  static const char* paths[] = {"auto", "tma", "trapezoid", "direct", "march", "strip"};
   static const char* bcs[] = {"periodic", "dirichlet", "external"};
   std::vector<int64_t> key{g.ndim, g.n[0], g.n[1], g.n[2], g.dtype, g.nf, s.kind, s.radius,
                            s.stages, c.path, c.tile_x, c.tile_y, c.k, nsteps, graph};
@@ -411,18 +456,20 @@ cudaError_t issue_stages(const Geom& g, const StencilDesc& s, const Choice& c,
   return cudaSuccess;
 }
 
-// Issue the launch sequence: ceil(nsteps/k) launches ping-ponging between out
+// Issue the launch sequence: the passes of count_passes, ping-ponging between out
 // and work so that the last one writes out.
 cudaError_t issue(const Geom& g, const StencilDesc& s, const Choice& c, const void* const* in,
                   void* const* out, void* const* work, int64_t nsteps, int* err, cudaStream_t st) {
-  if (s.stages >= 2 && c.path != kPathTrap)
+  if (s.stages >= 2 && c.path != kPathTrap && c.path != kPathStrip)
     return issue_stages(g, s, c, in, out, work, nsteps, err, st);
-  const int64_t L = (nsteps + c.k - 1) / c.k;
+  const int64_t L = count_passes(c, nsteps);
   const void* src[kMaxFields];
   for (int f = 0; f < g.nf; ++f) src[f] = in[f];
+  int64_t left = nsteps;
   for (int64_t j = 0; j < L; ++j) {
     StepArgs a = base_args(g, s, err, st);
-    a.ksteps = int(std::min<int64_t>(c.k, nsteps - j * c.k));
+    a.ksteps = int(next_depth(c, left));
+    left -= a.ksteps;
     a.tile_x = c.tile_x;
     a.tile_y = c.tile_y;
     const bool to_out = ((L - 1 - j) & 1) == 0;
@@ -435,6 +482,7 @@ cudaError_t issue(const Geom& g, const StencilDesc& s, const Choice& c, const vo
       case kPathTma: e = launch_tma(a, nullptr); break;
       case kPathTrap: e = launch_trap2d(a); break;
       case kPathMarch: e = launch_march(a); break;
+      case kPathStrip: e = launch_strip(a); break;
       default: e = launch_direct(a, nullptr); break;
     }
     if (e != cudaSuccess) return e;
@@ -535,9 +583,9 @@ lope_status prepare_apply(const lope_grid* grid, const lope_stencil* st, const v
     if (s.stages != 1)
       return fail(LOPE_ERR_UNSUPPORTED, "multi-stage schemes need a halo exchange per stage");
   }
-  if ((rs = resolve(g, s, in, cfg, nullptr, c)) != LOPE_OK) return rs;
-  *L = nsteps == 0 ? 0 : (nsteps + c->k - 1) / c->k;
-  const bool staged = s.stages >= 2 && c->path != kPathTrap;  // one launch per stage
+  if ((rs = resolve(g, s, in, nsteps, cfg, nullptr, c)) != LOPE_OK) return rs;
+  *L = count_passes(*c, nsteps);
+  const bool staged = s.stages >= 2 && c->path != kPathTrap && c->path != kPathStrip;  // one launch per stage
   if (staged) *L = nsteps * s.stages;
   return check_fields(g, in, out, work, staged ? nsteps >= 1 : *L >= 2, work_states(s), s.radius);
 }
@@ -828,7 +876,7 @@ lope_status gpu_tag_of(const char* gpu_name, std::string* out) {
 }
 
 bool choice_in_range(const Choice& c) {
-  return c.path >= kPathTma && c.path <= kPathMarch && c.tile_x >= 0 && c.tile_x <= 256 &&
+  return c.path >= kPathTma && c.path <= kPathStrip && c.tile_x >= 0 && c.tile_x <= 256 &&
          c.tile_y >= 0 && c.tile_y <= 256 && c.k >= 1 && c.k <= 8;
 }
 
@@ -1225,6 +1273,10 @@ lope_status lope_autotune(const lope_grid* grid, const lope_stencil* stencil,
   std::vector<lope_launch> cands;
   cands.push_back({kPathTma, 0, 0, 1, -1});
   if (g.ndim == 2) {
+    if (npts(g) >= (int64_t(1) << 20)) {  // strips: worth their pipeline fill from here on
+      StepArgs probe = base_args(g, stencil->s, nullptr, nullptr);
+      cands.push_back({kPathStrip, 0, 0, stencil->s.stages >= 2 ? 1 : strip_kmax_of(probe), -1});
+    }
     const int tiles[][2] = {{64, 32}, {128, 16}, {64, 16}, {32, 32}, {128, 32}};
     for (auto& t : tiles)
       for (int k : {1, 2, 3, 4, 6, 8}) cands.push_back({kPathTrap, t[0], t[1], k, -1});

@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "generic_kernels.cuh"
+#include "strip_kernels.cuh"
 #include "tma_kernels.cuh"
 
 namespace lope {
@@ -146,7 +147,7 @@ const char* type_name(int dtype) {
 template <int ND, int RR, int NFF, bool ST>
 struct UserOpHost {
   static constexpr int NDIM = ND, R = RR, NF = NFF;
-  static constexpr bool REDUCES = false, STAR = ST;
+  static constexpr bool REDUCES = false, STAR = ST, USER = true;
   Coef p[kUserParams];
   int* err;
 };
@@ -197,11 +198,12 @@ struct JitProgram {
 
   std::string source() const {
     std::string s;
-    s += "#include \"tma_device.cuh\"\n#include \"generic_device.cuh\"\n";
+    s += "#include \"tma_device.cuh\"\n#include \"generic_device.cuh\"\n#include \"strip_device.cuh\"\n";
     s += "namespace lope {\nstruct UserOp {\n";
     s += "  static constexpr int NDIM = " + std::to_string(ndim) + ", R = " + std::to_string(radius) +
          ", NF = " + std::to_string(nf) + ";\n";
-    s += std::string("  static constexpr bool REDUCES = false, STAR = ") + (star ? "true" : "false") + ";\n";
+    s += std::string("  static constexpr bool REDUCES = false, USER = true, STAR = ") +
+         (star ? "true" : "false") + ";\n";
     s += "  Coef p[" + std::to_string(kUserParams) + "];\n";
     s += "  int* err;\n";
     s += "  template <class C, class A>\n";
@@ -264,6 +266,24 @@ constexpr int tb2_index(bool wrap) { return kNumKernels + 8 + (wrap ? 1 : 0); }
 // follows at march_index(): 3D star functions of one field with FP32 / FP64
 // storage, for grids whose rows TMA cannot stage.
 constexpr int march_index() { return kNumKernels + 10; }
+// The register strips follow at strip_index(k): depths 4, 2 and 1 of 2D star
+// functions with FP32 / BF16 storage, for rows of whole vectors.
+constexpr int strip_index(int k) { return kNumKernels + 11 + (k == 4 ? 0 : k == 2 ? 1 : 2); }
+static_assert(kStripUserK == 4, "the depths compiled for user functions");
+template <class T, int RANK>
+constexpr bool jit_strip() {
+  return RANK == 2 && !std::is_same<T, double>::value;
+}
+template <class T, int R, int NF, int K>
+std::string strip_name() {
+  using Cfg = StripCfg<T, R, NF, K, 1>;
+  char buf[256];
+  std::snprintf(buf, sizeof(buf), "&lope::strip2d_kernel<lope::UserOp, %s, %d, 1, %d, %d, %d, true>",
+                std::is_same<T, float>::value ? "float" : "__nv_bfloat16", K, Cfg::D, Cfg::NWB,
+                Cfg::MINB);
+  return buf;
+}
+
 template <class T, int RANK, int NF>
 constexpr bool jit_march() {
   return RANK == 3 && NF == 1 && !std::is_same<T, __nv_bfloat16>::value;
@@ -284,7 +304,14 @@ template <int NF> constexpr int jit_tb2_ry() { return NF == 1 ? 8 : 2; }
 template <class T, int RANK, int R, int NF>
 void all_names(const JitProgram& jp, std::vector<std::string>* names) {
   kernel_names<T, RANK, R, NF>(jp, names);
-  names->resize(kNumKernels + 11);
+  names->resize(kNumKernels + 14);
+  if constexpr (jit_strip<T, RANK>()) {
+    if (jp.star) {
+      (*names)[strip_index(4)] = strip_name<T, R, NF, 4>();
+      (*names)[strip_index(2)] = strip_name<T, R, NF, 2>();
+      (*names)[strip_index(1)] = strip_name<T, R, NF, 1>();
+    }
+  }
   if (!jp.tma_ok()) return;
   if constexpr (jit_march<T, RANK, NF>()) {
     using CR = CaRunner<UserOpHost<RANK, R, NF, true>, T>;
@@ -602,6 +629,41 @@ cudaError_t run_march(JitProgram& jp, const StepArgs& a, int dtype) {
   }
 }
 
+// K sweeps on the register strips (strip_supported decided the grid).
+template <class T, int R, int NF, int K>
+cudaError_t run_strip_k(JitProgram& jp, const StepArgs& a, int dtype) {
+  using Host = UserOpHost<2, R, NF, true>;
+  using SR = StripRunner<Host, T, K, 1>;
+  CUfunction f = nullptr;
+  int occ = 1;
+  cudaError_t e = get_kernel(jp, dtype, strip_index(K), SR::SMEM, 32 * SR::Cfg::NWB, &f, &occ);
+  if (e != cudaSuccess) return e;
+  StripParams<Host, T> p;
+  std::memset(static_cast<void*>(&p), 0, sizeof(p));
+  for (int i = 0; i < kUserParams; ++i) p.op.p[i] = jp.prm[i];
+  p.op.err = a.err;
+  SR::params(a, occ, &p);
+  void* args[] = {&p};
+  return launch(f, (p.units + SR::Cfg::NWB - 1) / SR::Cfg::NWB, 32 * SR::Cfg::NWB, SR::SMEM, a.stream, args);
+}
+template <class T, int RANK, int R, int NF>
+cudaError_t run_strip(JitProgram& jp, const StepArgs& a, int dtype) {
+  if constexpr (jit_strip<T, RANK>()) {
+    if (!jp.star || !strip_vec(a)) return cudaErrorNotSupported;
+    switch (a.ksteps) {
+      case 4: return run_strip_k<T, R, NF, 4>(jp, a, dtype);
+      case 2: return run_strip_k<T, R, NF, 2>(jp, a, dtype);
+      case 1: return run_strip_k<T, R, NF, 1>(jp, a, dtype);
+      default: return cudaErrorNotSupported;
+    }
+  } else {
+    (void)jp;
+    (void)a;
+    (void)dtype;
+    return cudaErrorNotSupported;
+  }
+}
+
 template <class T, int RANK, int R, int NF>
 cudaError_t run_direct(JitProgram& jp, const StepArgs& a, int dtype) {
   using Host = UserOpHost<RANK, R, NF, true>;
@@ -699,6 +761,7 @@ cudaError_t jit_launch(const StepArgs& a, int path) {
     if (path == kPathTma) return run_tma<T, RANK, R, NF>(*jp, a, dtype);
     if (path == kPathTrap) return run_trap<T, RANK, R, NF>(*jp, a, dtype);
     if (path == kPathMarch) return run_march<T, RANK, R, NF>(*jp, a, dtype);
+    if (path == kPathStrip) return run_strip<T, RANK, R, NF>(*jp, a, dtype);
     return run_direct<T, RANK, R, NF>(*jp, a, dtype);
   });
 }

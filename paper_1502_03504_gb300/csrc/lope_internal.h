@@ -24,7 +24,7 @@ enum : int { kF64 = 0, kF32 = 1, kBF16 = 2 };
 // the neighbouring slab's planes (or rows) -- the destination of a halo
 // exchange between the slabs of a decomposed grid.
 enum : int { kPeriodic = 0, kDirichlet = 1, kExternal = 2 };
-enum : int { kPathAuto = 0, kPathTma = 1, kPathTrap = 2, kPathDirect = 3, kPathMarch = 4 };
+enum : int { kPathAuto = 0, kPathTma = 1, kPathTrap = 2, kPathDirect = 3, kPathMarch = 4, kPathStrip = 5 };
 
 // Device error codes written to the error flag.
 constexpr int kErrTimeout = 1;
@@ -112,6 +112,19 @@ cudaError_t launch_direct(const StepArgs& a, int* blocks);
 // sweeps).
 cudaError_t launch_march(const StepArgs& a);
 bool march_supported(const StepArgs& a);
+// Register strips (strip_device.cuh): ksteps sweeps of a 2D function per pass
+// (or one Runge-Kutta step), at depth strip_kmax_of or 4, 2, 1.
+cudaError_t launch_strip(const StepArgs& a);
+cudaError_t launch_strip_swe(const StepArgs& a);
+cudaError_t launch_strip_linear(const StepArgs& a);
+bool strip_supported(const StepArgs& a);
+int strip_kmax_of(const StepArgs& a);
+constexpr int kStripUserK = 4;  // depth of run-time compiled functions
+// Depths of the strips: the largest of a function (8, 6 or 4), then 4, 2, 1.
+__host__ __device__ inline int strip_next_depth(int kmax, int64_t left) {
+  if (left >= kmax) return kmax;
+  return left >= 4 && kmax > 4 ? 4 : left >= 2 && kmax > 2 ? 2 : 1;
+}
 // Run-time compiled local functions (jit.cu).
 struct JitProgram;
 lope_status jit_create(const char* body, int ndim, int radius, int nf, bool star,

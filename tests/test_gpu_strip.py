@@ -1,0 +1,158 @@
+"""Register strips (path 5): K sweeps of a 2D function per launch with every
+intermediate state in registers.
+
+Every sweep rounds to the storage precision, so the result must equal one
+sweep per launch on the direct kernel bitwise: at the edges of the strips (the
+valid width is 120 or 112 columns), of the chunks and of the grid, for rows of
+any pitch, periodic and Dirichlet sides with zero and non-zero values, every
+depth, odd sweep counts, box and star functions, several fields, both
+multi-stage schemes and run-time compiled functions.
+"""
+import numpy as np
+import pytest
+import torch
+
+import lope_inputs as LI
+from gpu_helpers import to_device
+from user_bodies import GRAY_SCOTT
+
+pytestmark = pytest.mark.gpu
+
+DIRECT, STRIP = 3, 5
+BCS = [([0, 0], None), ([1, 1], None), ([0, 1], [0.0, (0.5, -0.25)]), ([(1, 1), 0], [(0.3, 0.7), 0.0]),
+       ([1, 1], [(0.3, -0.2), (0.0, 0.5)])]
+FUNCS = {
+    "jacobi5": ([0.2], 1, 1, (8, 4, 2, 1)),
+    "star9r2": ([0.1], 2, 1, (4, 2, 1)),
+    "swe_cgrid": ([0.02, 1.0, 1.0], 1, 3, (6, 4, 2, 1)),
+    "swe_flux": ([0.02, 1.0, 0.5, 1.0], 1, 3, (4, 2, 1)),
+}
+
+
+def _run(L, g, st, f, T, launch):
+    o = L.apply(g, st, f, nsteps=T, launch=launch)
+    torch.cuda.synchronize()
+    L.sync_status()
+    return o
+
+
+def _fields(shape, dtype, nf, seed):
+    x = LI.swe_fields(seed, shape) if nf == 3 else [LI.uniform_field(seed, shape, k * 10 ** 6) for k in range(nf)]
+    return [to_device(a - 1.0 if nf == 3 and k == 0 else a, dtype)[0] for k, a in enumerate(x)]
+
+
+def _check(L, g, st, f, T, k):
+    ref = _run(L, g, st, f, T, L.Launch(DIRECT, 0, 0, 0, -1))
+    got = _run(L, g, st, f, T, L.Launch(STRIP, 0, 0, k, -1))
+    for a, b in zip(got, ref):
+        assert torch.equal(a, b), (g.shape, T, k)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("name", list(FUNCS))
+@pytest.mark.parametrize("shape", [(40, 4), (3, 120), (65, 124), (200, 112), (1030, 232), (17, 1000)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_strips_bitwise_equal_direct(lope, name, shape, dtype):
+    prm, halo, nf, depths = FUNCS[name]
+    st = lope.Stencil.builtin(name, *prm)
+    f = _fields(shape, dtype, nf, 1800)
+    for bc, bv in BCS:
+        g = lope.Grid(shape, dtype, halo=halo, nfields=nf).set_boundaries(bc, bv)
+        for k in depths:
+            _check(lope, g, st, f, k, k)
+    _check(lope, g, st, f, 2 * depths[0] + 3, depths[0])  # passes of several depths
+
+
+@pytest.mark.parametrize("name", list(FUNCS))
+@pytest.mark.parametrize("shape", [(5, 1), (9, 3), (65, 119), (130, 225), (70, 1001)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_strips_rows_of_any_pitch(lope, name, shape):
+    prm, halo, nf, depths = FUNCS[name]
+    st = lope.Stencil.builtin(name, *prm)
+    f = _fields(shape, "f32", nf, 1810)
+    for bc, bv in BCS:
+        if halo > 1 and shape[1] < halo and bc[1] == 0:
+            continue  # a periodic axis shorter than the radius is refused
+        g = lope.Grid(shape, "f32", halo=halo, nfields=nf).set_boundaries(bc, bv)
+        for k in depths:
+            _check(lope, g, st, f, k, k)
+
+
+def test_strips_weight_tables(lope):
+    rng = np.random.default_rng(1820)
+    shape = (90, 236)
+    for r in (1, 2):
+        w = rng.uniform(0.0, 0.08, (2 * r + 1, 2 * r + 1))
+        w[r, r] = 1.0 - (w.sum() - w[r, r])
+        star = np.zeros_like(w)
+        star[r], star[:, r] = w[r], w[:, r]
+        for table in (w, star):
+            st = lope.Stencil.linear(table)
+            for dtype in ("f32", "bf16"):
+                f = _fields(shape, dtype, 1, 1821)
+                for bc, bv in BCS:
+                    g = lope.Grid(shape, dtype, halo=r).set_boundaries(bc, bv)
+                    _check(lope, g, st, f, 7, 4)
+
+
+@pytest.mark.parametrize("scheme", ["rk2", "rk3"])
+@pytest.mark.parametrize("name", list(FUNCS))
+def test_strips_multi_stage(lope, name, scheme):
+    prm, halo, nf, _ = FUNCS[name]
+    st = lope.Stencil.builtin(name, *prm).set_scheme(scheme)
+    for shape in ((77, 124), (300, 232)):
+        for dtype in ("f32", "bf16"):
+            f = _fields(shape, dtype, nf, 1830)
+            for bc, bv in BCS:
+                g = lope.Grid(shape, dtype, halo=halo, nfields=nf).set_boundaries(bc, bv)
+                _check(lope, g, st, f, 3, 1)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_strips_run_time_compiled(lope, dtype):
+    prm = [1.0, 0.16, 0.08, 0.035, 0.065]
+    st = lope.Stencil.source(GRAY_SCOTT, ndim=2, radius=1, nfields=2, params=prm)
+    for shape in ((61, 124), (200, 360)):
+        f = _fields(shape, dtype, 2, 1840)
+        for bc, bv in BCS:
+            g = lope.Grid(shape, dtype, halo=1, nfields=2).set_boundaries(bc, bv)
+            for T, k in ((4, 4), (7, 4), (3, 2)):
+                _check(lope, g, st, f, T, k)
+
+
+def test_strips_default_plan_and_refusals(lope):
+    """Twelve sweeps or more take the strips; what they cannot run is refused."""
+    shape = (64, 132)
+    u = torch.rand(shape, device="cuda")
+    o, w = torch.empty_like(u), torch.empty_like(u)
+    st = lope.Stencil.builtin("jacobi5", 0.2)
+    g = lope.Grid(shape, "f32", halo=1)
+    plan, n = lope.plan(g, st, u, o, w, nsteps=23)
+    assert (plan.path, plan.tsteps, n) == (STRIP, 8, 5)  # 8 + 8 + 4 + 2 + 1
+    assert lope.plan(g, st, u, o, w, nsteps=11)[0].path != STRIP
+    ref = _run(lope, g, st, u, 23, lope.Launch(DIRECT, 0, 0, 0, -1))
+    assert torch.equal(_run(lope, g, st, u, 23, None), ref)
+    for bad in (3, 6, 16):
+        with pytest.raises(lope.LopeError, match="UNSUPPORTED"):
+            lope.apply(g, st, u, nsteps=23, launch=lope.Launch(STRIP, 0, 0, bad, -1))
+    d = torch.rand(shape, device="cuda", dtype=torch.float64)
+    with pytest.raises(lope.LopeError, match="UNSUPPORTED"):
+        lope.apply(lope.Grid(shape, "f64", halo=1), st, d, nsteps=4, launch=lope.Launch(STRIP, 0, 0, 4, -1))
+
+
+@pytest.mark.parametrize("shape", [(300, 200), (97, 203)], ids=lambda s: "x".join(map(str, s)))
+def test_strips_write_only_their_output(lope, shape):
+    n = int(np.prod(shape))
+    guard, sentinel = 4096, -7.0e30
+    u = torch.rand(shape, device="cuda")
+    keep = u.clone()
+    st = lope.Stencil.builtin("jacobi5", 0.2)
+    for bc in ([0, 0], [1, 1]):
+        g = lope.Grid(shape, "f32", halo=1).set_boundaries(bc)
+        bufs = [torch.full((n + 2 * guard,), sentinel, device="cuda") for _ in range(2)]
+        out, work = (b[guard:guard + n].view(shape) for b in bufs)
+        lope.apply(g, st, u, out=out, work=work, nsteps=13, launch=lope.Launch(STRIP, 0, 0, 8, -1))
+        torch.cuda.synchronize()
+        for b in bufs:
+            assert bool((b[:guard] == sentinel).all()) and bool((b[guard + n:] == sentinel).all())
+        assert torch.equal(u, keep)
