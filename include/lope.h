@@ -280,20 +280,22 @@ lope_status lope_tune_cache_load(const char* path, const char* gpu_name, int* lo
 
 /* Batched form: n independent grids of possibly different extents and
  * boundaries (same dtype, nfields and stencil) advanced nsteps each in one
- * persistent launch per call, replayed from a cached CUDA graph.  in/out/work
+ * launch of a cached CUDA graph per call: one persistent kernel (trapezoid
+ * tiles), or one kernel per pass over the whole batch (register strips).  in/out/work
  * hold n*nfields pointers, grid-major.  workspace is caller device memory of at
  * least lope_batch_workspace_size bytes (about 64 bytes per 64 x 64 tile of
- * the batch, plus the grid list); it holds the work list, the tile records,
- * the tile-claim counter and the inter-block barrier, and must stay untouched
- * between calls that reuse it.
+ * the batch, plus the grid list); it holds the work list
+ * and the inter-block barrier, and must stay untouched between calls that
+ * reuse it.
  * cfg may be NULL: the choice of the batch autotuner for this batch (see
  * lope_autotune_batch), else, for FP32 star functions of radius 1-2 (jacobi5,
- * star9r2, linear star tables), the two-sweep register tiles (cfg->path 1:
- * 64 x 64 tiles staged by plain loads, any row pitch, two sweeps per pass),
- * and the trapezoid tiles otherwise (cfg->path 2: 64 x 32 tiles, depth 4;
- * tile_x, tile_y and tsteps choose another shape and depth).  Errors as
- * lope_apply; LOPE_ERR_TIMEOUT is reported by lope_sync_status if a bounded
- * barrier wait gave up. */
+ * star9r2, linear star tables), the register strips (cfg->path 5: any row
+ * pitch, up to 8 sweeps per pass for radius 1, 4 for radius 2, tsteps chooses
+ * 8 / 4, 2 or 1; cfg->path 1 runs them two sweeps per pass), and the trapezoid
+ * tiles otherwise (cfg->path 2: 64 x 32 tiles, depth 4; tile_x, tile_y and
+ * tsteps choose another shape and depth).  Errors as lope_apply;
+ * LOPE_ERR_TIMEOUT is reported by lope_sync_status if a bounded barrier wait
+ * gave up. */
 lope_status lope_batch_workspace_size(int n, const lope_grid* const* grids,
                                       const lope_stencil* stencil, const lope_launch* cfg,
                                       size_t* bytes);
@@ -302,8 +304,8 @@ lope_status lope_apply_batch(int n, const lope_grid* const* grids, const lope_st
                              int64_t nsteps, const lope_launch* cfg, void* workspace,
                              size_t workspace_bytes, void* cuda_stream);
 
-/* Batch autotuner: times the batched launch over the two-sweep register tiles
- * (where they apply) and the trapezoid tiles of shapes {128, 64} x {32, 16}
+/* Batch autotuner: times the batched launch over the register strips (where
+ * they apply, from 2^20 points on) and the trapezoid tiles of shapes {128, 64} x {32, 16}
  * and temporal depths {1, 2, 4, 5} on the caller's buffers (out and work
  * are overwritten), stores the fastest for this batch (grid extents and
  * boundaries, dtype, stencil) and returns it in *best (*best_ms its time for

@@ -789,7 +789,7 @@ GraphKey adjoint_key(int kind, const lope_grid* grid, const lope_stencil* st,
 // ------------------------------------------------------------------ batch
 struct BatchPlan {
   std::vector<BatchGrid> host;
-  BatchGrid* pinned = nullptr;
+  void* pinned = nullptr;
   BatchPlanDev dev;
   cudaGraphExec_t exec = nullptr;
   int blocks = 0;
@@ -802,19 +802,40 @@ struct BatchPlan {
 std::mutex g_batch_mu;
 std::map<std::vector<int64_t>, std::shared_ptr<BatchPlan>> g_batch;
 
-// Batch workspace: the barrier and claim counters (256 B), the grid list, and
-// one record per tile of the two-sweep batched tiles (64 x 64 tiles).
+// Batch workspace: the barrier counter (256 B), the grid list, and
+// 64 bytes per 64 x 64 tile, which hold the unit lists of the strips (16 bytes
+// per grid and 16 more).
 size_t round256(size_t b) { return (b + 255) / 256 * 256; }
-int64_t batch_tb2_items(int n, const lope_grid* const* grids) {
-  int64_t items = 0;
-  for (int i = 0; i < n; ++i)
-    items += ((grids[i]->g.n[2] + kBatchTb2X - 1) / kBatchTb2X) *
-             ((grids[i]->g.n[1] + kBatchTb2Y - 1) / kBatchTb2Y);
-  return items;
-}
 size_t batch_ws_bytes(int n, const lope_grid* const* grids) {
-  return 256 + round256(size_t(n) * sizeof(BatchGrid)) +
-         round256(size_t(batch_tb2_items(n, grids)) * sizeof(BatchItem));
+  int64_t tiles = 0;
+  for (int i = 0; i < n; ++i)
+    tiles += ((grids[i]->g.n[2] + kBatchTileX - 1) / kBatchTileX) *
+             ((grids[i]->g.n[1] + kBatchTileY - 1) / kBatchTileY);
+  return 256 + round256(size_t(n) * sizeof(BatchGrid)) + round256(size_t(tiles) * 64);
+}
+
+// Rows per unit and first unit of every grid at depth k: about eight units per
+// resident warp when the batch is that large (uneven grids then balance
+// within a pass), else one, and never fewer rows than the pipeline's fill.
+int batch_strip_units(const std::vector<BatchGrid>& grids, int radius, int k, int64_t warps,
+                      int* chunk, int* first) {
+  const int valid = batch_strip_valid(radius, k);
+  auto strips = [&](const BatchGrid& g) { return int64_t((g.nx + valid - 1) / valid); };
+  int64_t rows = 0;
+  for (const BatchGrid& g : grids) rows += strips(g) * g.ny;
+  const int64_t fill = 2 * k * radius;
+  int64_t h = rows / (8 * warps);
+  if (h < 8 * fill) h = std::min<int64_t>(8 * fill, (rows + warps - 1) / warps);
+  h = std::max<int64_t>(h, fill);
+  *chunk = int(std::min<int64_t>(h, 1 << 20));
+  int64_t u = 0;
+  for (size_t i = 0; i < grids.size(); ++i) {
+    first[i] = int(u);
+    u += strips(grids[i]) * ((grids[i].ny + *chunk - 1) / *chunk);
+    if (u > int64_t(0x7fffffff)) return -1;
+  }
+  first[grids.size()] = int(u);
+  return int(u);
 }
 
 // Batch autotuner cache: the fastest (tile, depth) per batch signature (grid
@@ -913,8 +934,8 @@ bool parse_tune_line(const std::string& line, const std::string& gpu, bool* batc
   if (!(is >> colon >> c->path >> c->tile_x >> c->tile_y >> c->k) || colon != ":") return false;
   if (!choice_in_range(*c)) return false;
   if (*batch && !((c->path == kPathTrap && c->tile_x >= 8 && c->tile_y >= 1) ||
-                  (c->path == kPathTma && c->tile_x == kBatchTb2X && c->tile_y == kBatchTb2Y &&
-                   c->k == 2)))
+                  (c->path == kPathTma && c->tile_x == kBatchTileX && c->tile_y == kBatchTileY &&
+                   c->k == 2) || c->path == kPathStrip))
     return false;
   return true;
 }
@@ -1353,30 +1374,38 @@ lope_status lope_apply_batch(int n, const lope_grid* const* grids, const lope_st
     void* work1[1] = {work ? work[i] : nullptr};
     if ((rs = check_fields(grids[i]->g, in1, out1, work1, true)) != LOPE_OK) return rs;
   }
-  // The two-sweep register tiles (path 1: 64 x 64 tiles, two sweeps per
-  // pass) serve FP32 star functions of radius 1-2 (jacobi5, star9r2, linear
-  // star tables) and are the default there; other batches take the trapezoid
-  // tiles (path 2, 64 x 32, four sweeps per pass).  A choice remembered by the
-  // batch autotuner comes first; cfg overrides either.
-  const bool tb2_ok = dtype == kF32 && s.star && s.radius <= 2 &&
-                      (s.kind == kJacobi5 || s.kind == kStar9r2 || s.kind == kLinear);
-  Choice tuned = tb2_ok ? Choice{kPathTma, kBatchTb2X, kBatchTb2Y, 2} : Choice{kPathTrap, 64, 32, 4};
+  // The register strips (path 5; path 1 runs them two sweeps per pass) serve FP32
+  // star functions of radius 1-2 (jacobi5, star9r2, linear star tables) and are
+  // the default there; other batches take the trapezoid tiles (path 2, 64 x 32,
+  // four sweeps per pass).  A choice remembered by the batch autotuner comes
+  // first; cfg overrides either.
+  const bool strip_ok = dtype == kF32 && s.star && s.radius <= 2 &&
+                        (s.kind == kJacobi5 || s.kind == kStar9r2 || s.kind == kLinear);
+  StepArgs probe = base_args(grids[0]->g, s, nullptr, nullptr);
+  const int kmax = strip_kmax_of(probe);
+  Choice tuned = strip_ok ? Choice{kPathStrip, 0, 0, kmax} : Choice{kPathTrap, 64, 32, 4};
   if (!cfg || cfg->path == kPathAuto || cfg->tile_x <= 0 || cfg->tile_y <= 0 || cfg->tsteps <= 0) {
     std::lock_guard<std::mutex> lk(g_btune_mu);
     auto it = g_btune.find(batch_sig(n, grids, s));
-    if (it != g_btune.end()) tuned = it->second;
+    // (a loaded choice that the strips cannot run is ignored)
+    if (it != g_btune.end() && (it->second.path != kPathStrip ||
+                                (strip_ok && strip_next_depth(kmax, it->second.k) == it->second.k)))
+      tuned = it->second;
   }
   const int path = cfg && cfg->path != kPathAuto ? cfg->path : tuned.path;
-  if (path != kPathTma && path != kPathTrap)
-    return fail(LOPE_ERR_UNSUPPORTED, "the batched launch runs trapezoid (2) or two-sweep (1) tiles");
-  const int mode = path == kPathTma ? 1 : 0;
-  const int tx = mode ? kBatchTb2X : cfg && cfg->tile_x > 0 ? cfg->tile_x : tuned.tile_x;
-  const int ty = mode ? kBatchTb2Y : cfg && cfg->tile_y > 0 ? cfg->tile_y : tuned.tile_y;
-  const int k = mode ? 2 : cfg && cfg->tsteps > 0 ? cfg->tsteps : tuned.k;
-  if (tx < 8 || tx > 256 || ty < 1 || ty > 256 || k < 1 || k > 8)
+  if (path != kPathTma && path != kPathTrap && path != kPathStrip)
+    return fail(LOPE_ERR_UNSUPPORTED, "the batched launch runs trapezoid tiles (2) or strips (5, or 1)");
+  const int mode = path == kPathTrap ? 0 : 1;
+  const bool same = path == tuned.path;  // else the caller's path with the defaults of that path
+  const int tx = mode ? 0 : cfg && cfg->tile_x > 0 ? cfg->tile_x : same ? tuned.tile_x : 64;
+  const int ty = mode ? 0 : cfg && cfg->tile_y > 0 ? cfg->tile_y : same ? tuned.tile_y : 32;
+  const int k = path == kPathTma ? 2
+                : cfg && cfg->tsteps > 0 ? cfg->tsteps
+                : same ? tuned.k : mode ? kmax : 4;
+  if ((!mode && (tx < 8 || tx > 256 || ty < 1 || ty > 256)) || k < 1 || k > 8)
     return fail(LOPE_ERR_INVALID, "bad batch tile or depth");
-  if (mode && cfg && cfg->tsteps > 0 && cfg->tsteps != 2)
-    return fail(LOPE_ERR_UNSUPPORTED, "the two-sweep batched tiles run two sweeps per pass");
+  if (mode && cfg && cfg->path != kPathStrip && cfg->tsteps > 0 && cfg->tsteps != 2)
+    return fail(LOPE_ERR_UNSUPPORTED, "a depth other than 2 needs path 2 or 5 named");
   DevState* d = nullptr;
   lope_status rs = dev_state(&d);
   if (rs != LOPE_OK) return rs;
@@ -1425,19 +1454,37 @@ lope_status lope_apply_batch(int n, const lope_grid* const* grids, const lope_st
         b.bc[1][sd] = g.bc[2][sd];
         b.bval[1][sd] = g.bval[2][sd];
       }
-      b.tiles_x = (b.nx + tx - 1) / tx;
+      b.tiles_x = mode ? 0 : (b.nx + tx - 1) / tx;
       b.first_item = items;
-      items += b.tiles_x * ((b.ny + ty - 1) / ty);
+      if (!mode) items += b.tiles_x * ((b.ny + ty - 1) / ty);
     }
     if (take_alloc_failure()) return fail(LOPE_ERR_ALLOC, "allocation refused (fail_alloc option)");
-    cudaError_t e = cudaMallocHost(&plan->pinned, sizeof(BatchGrid) * n);
+    // what goes into the workspace: the grid list, then the strips' unit lists
+    const size_t gbytes = round256(sizeof(BatchGrid) * n);
+    const size_t bytes = gbytes + (mode ? round256(sizeof(int) * kStripDepths * size_t(n + 1)) : 0);
+    if (256 + bytes > batch_ws_bytes(n, grids)) return fail(LOPE_ERR_ALLOC, "batch workspace too small");
+    cudaError_t e = cudaMallocHost(&plan->pinned, bytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
+    std::memset(static_cast<void*>(plan->pinned), 0, bytes);
     std::memcpy(plan->pinned, plan->host.data(), sizeof(BatchGrid) * n);
+    plan->blocks = maxb;
+    plan->dev.passes = (nsteps + k - 1) / k;
+    if (mode) {
+      int* first = reinterpret_cast<int*>(reinterpret_cast<char*>(plan->pinned) + gbytes);
+      const int depths[kStripDepths] = {1, 2, 4, k > 4 ? k : 4};
+      for (int d2 = 0; d2 < kStripDepths; ++d2) {
+        const int u = batch_strip_units(plan->host, s.radius, depths[d2], int64_t(maxb) * 4,
+                                        &plan->dev.chunk[d2], first + size_t(d2) * (n + 1));
+        if (u < 0) return fail(LOPE_ERR_INVALID, "batch too large");
+        plan->dev.units[d2] = u;
+      }
+      plan->dev.passes = count_passes({kPathStrip, 0, 0, k}, nsteps);
+    } else {
+      plan->blocks = std::min(items, maxb);
+    }
     char* ws = static_cast<char*>(workspace);
     plan->dev.grids = reinterpret_cast<const BatchGrid*>(ws + 256);
-    plan->dev.items = reinterpret_cast<BatchItem*>(ws + 256 + round256(sizeof(BatchGrid) * n));
-    if (mode == 1 && items != batch_tb2_items(n, grids))
-      return fail(LOPE_ERR_INVALID, "batch tile count mismatch");
+    plan->dev.first = reinterpret_cast<const int*>(ws + 256 + gbytes);
     plan->dev.ngrids = n;
     plan->dev.nitems = items;
     plan->dev.tile_x = tx;
@@ -1445,28 +1492,22 @@ lope_status lope_apply_batch(int n, const lope_grid* const* grids, const lope_st
     plan->dev.ksteps = k;
     plan->dev.nsteps = nsteps;
     plan->dev.barrier = reinterpret_cast<unsigned int*>(ws);
-    plan->dev.claim = reinterpret_cast<unsigned long long*>(ws + 128);
     plan->dev.err = d->err;
     plan->dev.wait_ns = (unsigned long long)wait_ms * 1000000ull;
     plan->dev.skip_block = int(skip);
     plan->dev.mode = mode;
-    plan->blocks = std::min(items, maxb);
-    // Capture: descriptor upload, barrier reset, persistent kernel.
+    // Capture: descriptor upload and counter reset, persistent kernel.
     cudaGraph_t graph = nullptr;
     e = cudaStreamBeginCapture(d->capture, cudaStreamCaptureModeRelaxed);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
     g_capturing = true;
     g_captured = 0;
-    cudaError_t e1 = cudaMemcpyAsync(ws + 256, plan->pinned, sizeof(BatchGrid) * n,
-                                     cudaMemcpyHostToDevice, d->capture);
-    cudaError_t e2 = cudaMemsetAsync(ws, 0, 256, d->capture);
-    cudaError_t e3 = launch_batch(plan->dev, s, dtype, plan->blocks, d->capture);
+    const cudaError_t e1 = launch_batch(plan->dev, s, dtype, plan->blocks, plan->pinned, bytes, d->capture);
     g_capturing = false;
     e = cudaStreamEndCapture(d->capture, &graph);
-    if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e != cudaSuccess) {
+    if (e1 != cudaSuccess || e != cudaSuccess) {
       if (graph) cudaGraphDestroy(graph);
-      return cuda_fail(e3 != cudaSuccess ? e3 : e1 != cudaSuccess ? e1 : e2 != cudaSuccess ? e2 : e,
-                       "capturing the batched launch");
+      return cuda_fail(e1 != cudaSuccess ? e1 : e, "capturing the batched launch");
     }
     e = cudaGraphInstantiate(&plan->exec, graph, 0);
     cudaGraphDestroy(graph);
@@ -1496,7 +1537,18 @@ lope_status lope_autotune_batch(int n, const lope_grid* const* grids, const lope
   double bms = 1e300;
   lope_launch bl = {0, 0, 0, 0, 0};
   lope_status last = LOPE_OK;
-  std::vector<lope_launch> cands = {{kPathTma, kBatchTb2X, kBatchTb2Y, 2, -1}};
+  std::vector<lope_launch> cands;
+  {
+    // Strips from 2^20 points on; batches below fit in a few trapezoid tiles
+    // per block.
+    int64_t pts = 0;
+    for (int i = 0; i < n; ++i)
+      if (grids[i]) pts += npts(grids[i]->g);
+    if (pts >= (int64_t(1) << 20) && grids[0]) {
+      StepArgs probe = base_args(grids[0]->g, stencil->s, nullptr, nullptr);
+      cands.push_back({kPathStrip, 0, 0, strip_kmax_of(probe), -1});
+    }
+  }
   for (const auto& t : tiles)
     for (int k : {1, 2, 4, 5}) cands.push_back({kPathTrap, t[0], t[1], k, -1});
   for (const auto& c : cands) {

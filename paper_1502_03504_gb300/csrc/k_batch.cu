@@ -1,5 +1,6 @@
 // Batched form: many independent grids of uneven sizes advanced together by
-// one persistent, cooperatively launched kernel.
+// one persistent, cooperatively launched kernel (trapezoid tiles), or one kernel
+// per pass (register strips, below).
 //
 // The work list holds every (grid, tile) pair of the batch.  Each pass runs k
 // fused sweeps on every tile (trap.cuh), then all blocks meet at a grid-wide
@@ -13,7 +14,7 @@
 #include <algorithm>
 #include <type_traits>
 
-#include "tma_device.cuh"
+#include "strip_kernels.cuh"
 #include "trap.cuh"
 
 namespace lope {
@@ -21,6 +22,7 @@ namespace lope {
 namespace {
 
 constexpr int kBatchThreads = 256;
+constexpr int kBatchWarps = 4, kBatchRing = 8;  // strips: warps per block, staged rows per warp
 
 __device__ __forceinline__ bool grid_sync(unsigned int* bar, unsigned int target, int* err,
                                           volatile int* s_abort, unsigned long long wait_ns,
@@ -117,318 +119,81 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(Op op, BatchPlanDe
   }
 }
 
-// ------------------------------------------------------------------ two sweeps per pass
-// The batched form of the two-sweep 2D tiles (tma2d_tb2_kernel), for FP32 grids
-// of any row pitch: a 64 x TY tile is staged into shared memory with a 2R-row
-// / 4-column halo by 4-byte asynchronous copies (cp.async; the grids' rows need
-// not be 16-byte aligned, as TMA would require), the boundary rule applied as
-// each cell is staged (rows first: the Dirichlet value, stored directly, or
-// the wrapped row; then columns likewise); the first sweep u1 is computed on
-// the tile and its R-wide ring and held at the side's Dirichlet value past a
-// Dirichlet side; the second sweep writes the tile.
-//
-// Two staging boxes alternate: the copies of the next tile are issued before
-// the first sweep of the current one, so they have a whole tile's sweeps to
-// land.  Tiles are claimed one at a time from a counter, two ahead of the
-// tile being swept, and each claimed tile's 64-byte record (BatchItem) is
-// read while the current tile's second sweep runs.  A pass (two sweeps, or
-// one for the last of an odd count) covers every tile of every grid; passes
-// are separated by the bounded grid-wide barrier, whose acquire orders the
-// next pass's copies after every block's stores.  All threads of a block run
-// the same control flow, so its barriers cannot strand a thread.
-template <int R>
-struct BatchTb2Geom {
-  static constexpr int TX = 64, H = 2 * R, CW = 4, W = TX + 2 * CW;  // box columns -4..TX+3
-  static constexpr int W1 = TX + 4;                                   // u1 columns -2..TX+1
-  static constexpr __host__ __device__ int box_floats(int ty) { return (ty + 2 * H) * W; }
-  static constexpr __host__ __device__ int u1_floats(int ty) { return (ty + 2 * R) * W1; }
-};
+// ------------------------------------------------------------------ strips
+// FP32 star functions: the register strips (strip_device.cuh) over every grid
+// of the batch.  A pass advances every grid by the same depth K (the plan's
+// depth, then 4, 2 and 1 for what is left of the sweep count) and is one launch
+// with one unit (a strip's chunk of rows of one grid) per warp; the block
+// scheduler balances uneven grids.  Rows of any pitch (aligned grids stage
+// whole vectors).  A persistent kernel whose warps claimed units from a counter
+// kept about 45 registers of its loop alive across the march and spilled it
+// (512 grids of sides 64..2048, jacobi5 x20, 5.9e8 points: 9.5 ms, with all
+// depths in one kernel 11.6 ms; this form 5.57 ms, the two-sweep shared-memory
+// tiles it replaced 12.5 ms).  Bound by instruction issue: 16 grids of 4096^2
+// run 3.6e12 updates/s at depth 8; odd widths (element copies and stores)
+// and Dirichlet sides (masks) cost a quarter to a third.
 
-// Fill the tile records of the two-sweep batched tiles from the grid list.
-__global__ void batch_items_kernel(const BatchGrid* grids, int ngrids, int nitems, int tx, int ty,
-                                   BatchItem* items) {
-  for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < nitems; it += gridDim.x * blockDim.x) {
-    const BatchGrid& g = grids[find_grid(grids, ngrids, it)];
-    const int t = it - g.first_item;
-    BatchItem b;
-    b.in = static_cast<const float*>(g.in);
-    b.out = static_cast<float*>(g.out);
-    b.work = static_cast<float*>(g.work);
-    b.nx = g.nx;
-    b.ny = g.ny;
-    b.x0 = (t % g.tiles_x) * tx;
-    b.y0 = (t / g.tiles_x) * ty;
-    b.bc = (g.bc[0][0] & 255) | (g.bc[0][1] & 255) << 8 | (g.bc[1][0] & 255) << 16 |
-           (g.bc[1][1] & 255) << 24;
-    b.vy0 = float(g.bval[0][0]);
-    b.vy1 = float(g.bval[0][1]);
-    b.vx0 = float(g.bval[1][0]);
-    b.vx1 = float(g.bval[1][1]);
-    b.pad = 0;
-    items[it] = b;
+// The grid of unit `item`: first[i] is the first unit of grid i (ascending).
+// All lanes probe 32 positions of the list at once.
+__device__ __forceinline__ int find_grid_warp(const int* first, int n, int item) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, len = n;
+  while (len > 1) {
+    const int step = (len + 31) / 32, i = lane * step;
+    const unsigned le = __ballot_sync(0xffffffffu, i < len && first[lo + (i < len ? i : 0)] <= item);
+    const int j = (__popc(le) - 1) * step;
+    lo += j;
+    len = min(step, len - j);
   }
+  return lo;
 }
 
-template <class Op, int TY, int RY>
-__global__ void __launch_bounds__(32 * (TY / RY), 3) batch_tb2_kernel(Op op, BatchPlanDev p) {
-  using G = BatchTb2Geom<Op::R>;
-  constexpr int TX = G::TX, R = Op::R, H = G::H, CW = G::CW, W = G::W, W1 = G::W1;
-  static_assert(Op::NF == 1 && Op::STAR && R <= 2, "radius <= 2 star function of one field");
-  constexpr int BH = TY + 2 * H, NW = TY / RY, NT = 32 * NW;
-  constexpr int NC = RY + 2 * R, BOXN = G::box_floats(TY);
-  constexpr int NRING = 2 * R * 32 + 2 * TY;
+// One pass of depth K over the batch; pass 0 reads in, pass q > 0 what pass q-1
+// wrote.
+template <class Op, int K>
+__global__ void __launch_bounds__(32 * kBatchWarps, 4)
+    batch_strip_kernel(const __grid_constant__ Op op, const __grid_constant__ BatchPlanDev p,
+                       int64_t pass) {
+  using G = StripGeom<float, Op::R, K>;
+  constexpr int D = strip_depth_index(K);
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* const boxes = reinterpret_cast<float*>(smem_raw);  // two staging boxes
-  float* const u1 = boxes + 2 * BOXN;
-  // Tile records: the tile being swept, the next one (staged during this
-  // tile's sweeps) and the one after (fetched during the second sweep).
-  __shared__ __align__(16) BatchItem s_rec[3];
-  __shared__ volatile int s_abort;
-  __shared__ int s_claim;
-  const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
-  const int cx2 = lane * 2, cy0 = warp * RY;
-  if (tid == 0) s_abort = 0;
-  __syncthreads();
-  // Threads 0-3 copy the four 16-byte quarters of a record into slot `sl`
-  // (asynchronously; the copy lands by the next wait).
-  auto fetch_rec = [&](int item, int sl) {
-    if (item >= 0 && tid < 4) {
-      const uint32_t d = smem_u32(&s_rec[sl]) + 16u * unsigned(tid);
-      const char* src = reinterpret_cast<const char*>(p.items + item) + 16 * tid;
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  const int warp = threadIdx.x / 32;
+  const int u = blockIdx.x * kBatchWarps + warp;
+  if (u >= p.units[D]) return;
+  unsigned char* ring = smem_raw + warp * (kBatchRing * G::ROWB);
+  const int* first = p.first + size_t(D) * (p.ngrids + 1);
+  const int gi = find_grid_warp(first, p.ngrids, u);
+  const BatchGrid& b = p.grids[gi];
+  const bool to_out = ((p.passes - 1 - pass) & 1) == 0;
+  const float* in[1] = {static_cast<const float*>(pass == 0 ? b.in : to_out ? b.work : b.out)};
+  float* out[1] = {static_cast<float*>(to_out ? b.out : b.work)};
+  StripGrid g;
+  g.nx = b.nx;
+  g.ny = b.ny;
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int sd = 0; sd < 2; ++sd) {
+      g.bc[a][sd] = b.bc[a][sd];
+      g.bval[a][sd] = b.bval[a][sd];
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
+  const int strips = (g.nx + G::VALID - 1) / G::VALID;
+  const int t = u - first[gi], c = t / strips, s = t - c * strips;
+  const int y0 = c * p.chunk[D], y1 = min(g.ny, y0 + p.chunk[D]);
+  if (g.nx % kStripV == 0)
+    Strip<Op, float, K, 1, kBatchRing, true>::run(op, in, out, g, s * G::VALID, y0, y1, ring, nullptr);
+  else
+    Strip<Op, float, K, 1, kBatchRing, false>::run(op, in, out, g, s * G::VALID, y0, y1, ring, nullptr);
+}
 
-  const int64_t passes = (p.nsteps + 1) / 2;
-  for (int64_t pass = 0; pass < passes; ++pass) {
-    const int kp = (pass == passes - 1 && (p.nsteps & 1)) ? 1 : 2;
-    const bool to_out = ((passes - 1 - pass) & 1) == 0;
-    // Each block claims until its first claim past the list and then once
-    // more (the claims run two tiles ahead), so each pass takes exactly
-    // nitems + 2 * gridDim.x claims and pass `pass` starts from
-    // pass * (nitems + 2 * gridDim.x).
-    const unsigned long long pbase =
-        (unsigned long long)pass * (unsigned long long)(p.nitems + 2 * int(gridDim.x));
-    auto claim_raw = [&]() { return atomicAdd(p.claim, 1ull) - pbase; };
-    auto valid = [&](unsigned long long v) { return v < (unsigned long long)p.nitems ? int(v) : -1; };
-    // Stage the tile of record `t` into `box`: warp w takes box rows w,
-    // w + NW, ...; lane l the box columns l, l + 32, l + 64.  A tile whose box
-    // lies inside its grid copies every cell; elsewhere the row rule is
-    // decided once per row and the column rule once per column, rows (the
-    // slower axis) first.  Ends with a commit, so each tile's copies form
-    // one group.
-    auto load = [&](const BatchItem& t, float* box) {
-      const uint32_t sbox = smem_u32(box);
-      const float* src = pass == 0 ? t.in : (to_out ? t.work : t.out);
-      const int nx = t.nx, ny = t.ny, x0 = t.x0, y0 = t.y0;
-      if (x0 >= CW && x0 + TX + CW <= nx && y0 >= H && y0 + TY + H <= ny) {
-        // a box row is a run of consecutive cells: 16- or 8-byte copies where
-        // the run's first cell is so aligned (box rows are 16-byte aligned)
-        const float* r0 = src + int64_t(y0 - H + warp) * nx + (x0 - CW);
-        const int64_t step = int64_t(NW) * nx;
-        uint32_t d = sbox + 4u * unsigned(warp * W);
-        static_assert(W % 4 == 0 && W / 4 <= 32 && W / 2 <= 64 && W <= 96, "box row copies");
-#pragma unroll 4
-        for (int br = warp; br < BH; br += NW, r0 += step, d += 4u * NW * W) {
-          const unsigned mis = unsigned(reinterpret_cast<uintptr_t>(r0)) & 15u;
-          if (mis == 0) {
-            if (lane < W / 4) cp_async_16(d + 16u * lane, r0 + 4 * lane);
-          } else if ((mis & 7u) == 0) {
-            cp_async_elem<8>(d + 8u * lane, r0 + 2 * lane);
-            if (lane < W / 2 - 32) cp_async_elem<8>(d + 8u * (lane + 32), r0 + 2 * (lane + 32));
-          } else {
-            cp_async_elem<4>(d + 4u * lane, r0 + lane);
-            cp_async_elem<4>(d + 4u * (lane + 32), r0 + lane + 32);
-            if (lane < W - 64) cp_async_elem<4>(d + 4u * (lane + 64), r0 + lane + 64);
-          }
-        }
-      } else {
-        const int bcy0 = t.bc & 255, bcy1 = (t.bc >> 8) & 255;
-        const int bcx0 = (t.bc >> 16) & 255, bcx1 = (t.bc >> 24) & 255;
-        int gcol[3];
-        float cval[3];
-        bool cfix[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          int gx = x0 - CW + lane + 32 * k;
-          cfix[k] = false;
-          cval[k] = 0.f;
-          if (gx < 0 || gx >= nx) {
-            const bool lo = gx < 0;
-            if ((lo ? bcx0 : bcx1) == kDirichlet) {
-              cfix[k] = true;
-              cval[k] = lo ? t.vx0 : t.vx1;
-            }
-            gx = wrap(gx, nx);
-          }
-          gcol[k] = gx;
-        }
-        for (int br = warp; br < BH; br += NW) {
-          int gy = y0 - H + br;
-          bool rfix = false;
-          float rval = 0.f;
-          if (gy < 0 || gy >= ny) {
-            const bool lo = gy < 0;
-            if ((lo ? bcy0 : bcy1) == kDirichlet) {
-              rfix = true;
-              rval = lo ? t.vy0 : t.vy1;
-            }
-            gy = wrap(gy, ny);
-          }
-          const float* row = src + int64_t(gy) * nx;
-#pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            if (lane + 32 * k >= W) break;
-            const int at = br * W + lane + 32 * k;
-            if (rfix) box[at] = rval;
-            else if (cfix[k]) box[at] = cval[k];
-            else cp_async_elem<4>(sbox + 4u * unsigned(at), row + gcol[k]);
-          }
-        }
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    // Prologue: the first tile claimed, its record read and its box staged;
-    // the second claimed and its record fetched.
-    if (tid == 0) s_claim = valid(claim_raw());
-    __syncthreads();
-    int cur = s_claim;
-    fetch_rec(cur, 0);
-    cp_async_wait_all();
-    __syncthreads();  // the record is visible; every thread has read s_claim
-    if (tid == 0) s_claim = valid(claim_raw());
-    if (cur >= 0) load(s_rec[0], boxes);
-    __syncthreads();
-    int nxt = s_claim;
-    fetch_rec(nxt, 1);
-    int a = 0, b = 1, c = 2, buf = 0;
-    while (cur >= 0) {
-      cp_async_wait_all();
-      __syncthreads();  // this tile's box and the next record have landed; u1 is free
-      // the next tile's copies go to the other box, free since the barrier
-      // after the previous tile's first sweep
-      if (nxt >= 0) load(s_rec[b], boxes + (buf ^ 1) * BOXN);
-      unsigned long long v = 0;
-      if (tid == 0) v = claim_raw();  // the tile after next; published after the first sweep
-      const BatchItem& t = s_rec[a];
-      const float* box = boxes + buf * BOXN;
-      const int nx = t.nx, ny = t.ny, x0 = t.x0, y0 = t.y0;
-      const bool edge = x0 < CW || x0 + TX + CW > nx || y0 < H || y0 + TY + H > ny;
-      auto sweep1 = [&](auto edge_tag) {
-        constexpr bool EDGE = decltype(edge_tag)::value;
-        // Cells past a Dirichlet side keep its value: tile rows outside
-        // [row_lo, row_hi) and columns outside [col_lo, col_hi) (rows first,
-        // then columns, the order of the boundary rule).
-        constexpr int kFar = 1 << 30;
-        int row_lo = -kFar, row_hi = kFar, col_lo = -kFar, col_hi = kFar;
-        float vy0 = 0.f, vy1 = 0.f, vx0 = 0.f, vx1 = 0.f;
-        if constexpr (EDGE) {
-          if ((t.bc & 255) == kDirichlet) row_lo = -y0;
-          if (((t.bc >> 8) & 255) == kDirichlet) row_hi = ny - y0;
-          if (((t.bc >> 16) & 255) == kDirichlet) col_lo = -x0;
-          if (((t.bc >> 24) & 255) == kDirichlet) col_hi = nx - x0;
-          vy0 = t.vy0;
-          vy1 = t.vy1;
-          vx0 = t.vx0;
-          vx1 = t.vx1;
-        }
-        auto cell = [&](float v, int tc) { return tc < col_lo ? vx0 : tc >= col_hi ? vx1 : v; };
-        auto mask = [&](F2 v, int tr, int tc) {
-          if (tr < row_lo) return F2::make(vy0, vy0);
-          if (tr >= row_hi) return F2::make(vy1, vy1);
-          return F2::make(cell(v.lo(), tc), cell(v.hi(), tc + 1));
-        };
-        F2 col[NC];
-#pragma unroll
-        for (int k = 0; k < NC; ++k) col[k] = ld_pair(box + (H - R + cy0 + k) * W + CW + cx2);
-#pragma unroll
-        for (int r = 0; r < RY; ++r) {
-          PairAcc<float, TX, TY, R, 1, NC> acc;
-          acc.b[0] = box + (H + cy0 + r) * W + CW + cx2;
-          acc.col = &col;
-          acc.r = r;
-          acc.g = 0;
-          F2 o[1];
-          F2 unused(0.f);
-          op(acc, o, unused);
-          F2 v = o[0];
-          if constexpr (EDGE) v = mask(v, cy0 + r, cx2);
-          st_pair_f(u1 + (R + cy0 + r) * W1 + 2 + cx2, v);
-        }
-        for (int q = tid; q < NRING; q += NT) {
-          int tr, tc;
-          if (q < 2 * R * 32) {
-            const int row = q >> 5;
-            tr = row < R ? row - R : TY + row - R;
-            tc = (q & 31) * 2;
-          } else {
-            const int d = q - 2 * R * 32;
-            tr = d >> 1;
-            tc = (d & 1) ? TX : -2;
-          }
-          Smem2Acc<float, W> acc{box + (H + tr) * W + CW + tc};
-          F2 o[1];
-          F2 unused(0.f);
-          op(acc, o, unused);
-          F2 v = o[0];
-          if constexpr (EDGE) v = mask(v, tr, tc);
-          st_pair_f(u1 + (R + tr) * W1 + 2 + tc, v);
-        }
-      };
-      if (edge) sweep1(BoolTag<true>());
-      else sweep1(BoolTag<false>());
-      if (tid == 0) s_claim = valid(v);
-      __syncthreads();  // u1 complete; s_claim published; this box is free
-      const int nn = s_claim;
-      fetch_rec(nn, c);  // the record slot of the previous tile, read before the barrier above
-      float* const out = to_out ? t.out : t.work;
-      const int ox = x0 + cx2, oy = y0 + cy0;
-      auto put = [&](int r, F2 v) {
-        const int gy = oy + r;
-        if (gy >= ny || ox >= nx) return;
-        float* d = out + int64_t(gy) * nx + ox;
-        if (ox + 1 < nx && (reinterpret_cast<uintptr_t>(d) & 7) == 0) {
-          st_pair(d, v);
-        } else {
-          d[0] = v.lo();
-          if (ox + 1 < nx) d[1] = v.hi();
-        }
-      };
-      if (kp == 1) {  // a one-sweep pass: u1 is the result
-#pragma unroll
-        for (int r = 0; r < RY; ++r) put(r, ld_pair(u1 + (R + cy0 + r) * W1 + 2 + cx2));
-      } else {
-        F2 col[NC];
-#pragma unroll
-        for (int k = 0; k < NC; ++k) col[k] = ld_pair(u1 + (cy0 + k) * W1 + 2 + cx2);
-#pragma unroll
-        for (int r = 0; r < RY; ++r) {
-          PairAcc<float, TX, TY, R, 1, NC> acc;
-          acc.b[0] = u1 + (R + cy0 + r) * W1 + 2 + cx2;
-          acc.col = &col;
-          acc.r = r;
-          acc.g = 0;
-          F2 o[1];
-          F2 unused(0.f);
-          op(acc, o, unused);
-          put(r, o[0]);
-        }
-      }
-      cur = nxt;
-      nxt = nn;
-      const int a0 = a;
-      a = b;
-      b = c;
-      c = a0;
-      buf ^= 1;
-    }
-    cp_async_wait_all();
-    const bool arrive = !(pass == 0 && int(blockIdx.x) == p.skip_block);
-    if (pass + 1 < passes &&
-        !grid_sync(p.barrier, unsigned(pass + 1) * gridDim.x, p.err, &s_abort, p.wait_ns, arrive))
-      return;
-  }
+// Copy the plan's descriptors from page-locked host memory into the workspace
+// and zero its counters.  A kernel, not copy and memset nodes: those belong to
+// the allocation that held the workspace when the graph was made, and a replay
+// after the caller freed and allocated it again at the same address is invalid.
+__global__ void batch_upload_kernel(const uint4* src, uint4* dst, int64_t n16, uint4* counters) {
+  const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (i < 16) counters[i] = make_uint4(0, 0, 0, 0);
+  if (i < n16) dst[i] = src[i];
 }
 
 template <class Op, class T, class Tile> struct BatchRunner {
@@ -488,61 +253,36 @@ auto with_tile(int tx, int ty, int k, F&& f) {
   return f(TileAny());
 }
 
-// Two-sweep register tiles: 8 warps of 8 rows on 64 x 64 tiles, three blocks
-// per SM, each with two staging boxes (measured on the 512-grid workload:
-// 12.3 ms for 20 sweeps against 15.0 ms on 64 x 128 tiles with two blocks of
-// 8 warps of 16 rows, and 14.4 ms with two blocks of 16 warps of 8 rows).
-constexpr int kTb2RY = 8, kTb2Threads = 32 * (kBatchTb2Y / kTb2RY);
-
-template <class Op>
-size_t tb2_smem() {
-  using G = BatchTb2Geom<Op::R>;
-  return size_t(2 * G::box_floats(kBatchTb2Y) + G::u1_floats(kBatchTb2Y)) * 4;
+template <class Op, int K>
+cudaError_t launch_strip_pass(const Op& op, const BatchPlanDev& p, int64_t pass, cudaStream_t st) {
+  constexpr size_t SMEM = size_t(kBatchWarps) * kBatchRing * StripGeom<float, Op::R, K>::ROWB;
+  const int blocks = (p.units[strip_depth_index(K)] + kBatchWarps - 1) / kBatchWarps;
+  batch_strip_kernel<Op, K><<<blocks, 32 * kBatchWarps, SMEM, st>>>(op, p, pass);
+  count_launches(1);
+  return cudaGetLastError();
 }
 
 template <class Op>
-struct BatchTb2Runner {
-  static auto kernel() { return &batch_tb2_kernel<Op, kBatchTb2Y, kTb2RY>; }
-  static int max_blocks() {
-    if (cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(tb2_smem<Op>())) != cudaSuccess)
-      return 0;
-    int occ = 0, dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel(), kTb2Threads, tb2_smem<Op>()) !=
-        cudaSuccess)
-      return 0;
-    return occ * sms;
-  }
-  static cudaError_t launch(const Op& op, const BatchPlanDev& p, int blocks, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(tb2_smem<Op>()));
+cudaError_t launch_strips(const Op& op, const BatchPlanDev& p, cudaStream_t st) {
+  int64_t pass = 0;
+  for (int64_t left = p.nsteps; left > 0; ++pass) {
+    const int k = strip_next_depth(p.ksteps, left);
+    cudaError_t e = cudaErrorNotSupported;
+    if constexpr (strip_kmax(1, Op::R, true) >= 8) {
+      if (k == 8) e = launch_strip_pass<Op, 8>(op, p, pass, st);
+    }
+    if (k == 4) e = launch_strip_pass<Op, 4>(op, p, pass, st);
+    if (k == 2) e = launch_strip_pass<Op, 2>(op, p, pass, st);
+    if (k == 1) e = launch_strip_pass<Op, 1>(op, p, pass, st);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(kTb2Threads);
-    cfg.dynamicSmemBytes = tb2_smem<Op>();
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    // the tile records first (one thread per tile), then the persistent kernel
-    batch_items_kernel<<<(p.nitems + 255) / 256, 256, 0, st>>>(p.grids, p.ngrids, p.nitems,
-                                                               kBatchTb2X, kBatchTb2Y, p.items);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    e = cudaLaunchKernelEx(&cfg, kernel(), op, p);
-    count_launches(2);
-    return e;
+    left -= k;
   }
-};
+  return cudaSuccess;
+}
 
-// Local functions of the two-sweep batched tiles: the 5-point Jacobi, the
-// 9-point radius-2 star, and linear star tables of radius 1 or 2.
-template <class F> cudaError_t with_tb2_op(const StencilDesc& s, F&& f) {
+// Local functions of the batched strips: the 5-point Jacobi, the 9-point
+// radius-2 star, and linear star tables of radius 1 or 2.
+template <class F> cudaError_t with_strip_op(const StencilDesc& s, F&& f) {
   if (s.kind == kJacobi5) return f(OpJacobi5{s.prm[0]});
   if (s.kind == kStar9r2) return f(OpStar9r2{s.prm[0]});
   if (s.kind == kLinear && s.star && s.ndim == 2 && s.radius == 1) {
@@ -580,12 +320,27 @@ template <class T> int max_blocks_t(const StencilDesc& s, int tx, int ty, int k)
 
 }  // namespace
 
+// Columns a strip of depth k advances (the cut of the batch's grids).
+int batch_strip_valid(int radius, int k) {
+  const int hl = (k * radius + kStripV - 1) / kStripV;
+  return (32 - 2 * hl) * kStripV;
+}
+
 cudaError_t launch_batch(const BatchPlanDev& p, const StencilDesc& s, int dtype, int blocks,
-                         cudaStream_t st) {
+                         const void* pinned, size_t bytes, cudaStream_t st) {
+  {
+    const int64_t n16 = int64_t((bytes + 15) / 16);
+    batch_upload_kernel<<<int((std::max<int64_t>(n16, 16) + 255) / 256), 256, 0, st>>>(
+        static_cast<const uint4*>(pinned), reinterpret_cast<uint4*>(const_cast<BatchGrid*>(p.grids)), n16,
+        reinterpret_cast<uint4*>(p.barrier));
+    count_launches(1);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   if (p.mode == 1) {
     if (dtype != kF32) return cudaErrorNotSupported;
-    return with_tb2_op(s, [&](auto op) {
-      return BatchTb2Runner<decltype(op)>::launch(op, p, blocks, st);
+    return with_strip_op(s, [&](auto op) {
+      return launch_strips(op, p, st);
     });
   }
   if (!(s.kind == kJacobi5 || (s.kind == kLinear && s.star && s.ndim == 2 && s.radius == 1)))
@@ -601,14 +356,11 @@ cudaError_t launch_batch(const BatchPlanDev& p, const StencilDesc& s, int dtype,
 int batch_max_blocks(const StencilDesc& s, int dtype, int tile_x, int tile_y, int ksteps,
                      int mode) {
   if (mode == 1) {
-    if (dtype != kF32 || tile_x != kBatchTb2X || tile_y != kBatchTb2Y || ksteps < 1 || ksteps > 2)
+    if (dtype != kF32 || (ksteps != strip_kmax(1, s.radius, true) && ksteps != 4 && ksteps != 2 && ksteps != 1))
       return 0;
-    int b = 0;
-    with_tb2_op(s, [&](auto op) {
-      b = BatchTb2Runner<decltype(op)>::max_blocks();
-      return cudaSuccess;
-    });
-    return b;
+    // resident blocks (the units are cut for them; nothing waits on another)
+    const cudaError_t e = with_strip_op(s, [](auto) { return cudaSuccess; });
+    return e == cudaSuccess ? 4 * strip_sms() : 0;
   }
   if (!(s.kind == kJacobi5 || (s.kind == kLinear && s.star && s.ndim == 2 && s.radius == 1)))
     return 0;

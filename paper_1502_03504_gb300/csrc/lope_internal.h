@@ -120,11 +120,6 @@ cudaError_t launch_strip_linear(const StepArgs& a);
 bool strip_supported(const StepArgs& a);
 int strip_kmax_of(const StepArgs& a);
 constexpr int kStripUserK = 4;  // depth of run-time compiled functions
-// Depths of the strips: the largest of a function (8, 6 or 4), then 4, 2, 1.
-__host__ __device__ inline int strip_next_depth(int kmax, int64_t left) {
-  if (left >= kmax) return kmax;
-  return left >= 4 && kmax > 4 ? 4 : left >= 2 && kmax > 2 ? 2 : 1;
-}
 // Run-time compiled local functions (jit.cu).
 struct JitProgram;
 lope_status jit_create(const char* body, int ndim, int radius, int nf, bool star,
@@ -167,40 +162,41 @@ struct BatchGrid {
   int tiles_x;
   int first_item;     // index of this grid's first tile in the global item list
 };
-// One tile of the two-sweep batched tiles (mode 1), 64 bytes: everything a
-// block needs to stage and sweep it, read with four 16-byte loads.  Filled
-// on the device from the grid list at the start of each batched launch.
-struct __align__(16) BatchItem {
-  const float* in;
-  float* out;
-  float* work;
-  int nx, ny, x0, y0;
-  int bc;             // side kinds, 8 bits each: y low, y high, x low, x high
-  float vy0, vy1, vx0, vx1;
-  int pad;
-};
+// Depths of the strips: the largest of a function (8, 6 or 4), then 4, 2, 1.
+__host__ __device__ inline int strip_next_depth(int kmax, int64_t left) {
+  if (left >= kmax) return kmax;
+  return left >= 4 && kmax > 4 ? 4 : left >= 2 && kmax > 2 ? 2 : 1;
+}
+__host__ __device__ constexpr int strip_depth_index(int k) { return k == 1 ? 0 : k == 2 ? 1 : k == 4 ? 2 : 3; }
+constexpr int kStripDepths = 4;
+
 struct BatchPlanDev {
   const BatchGrid* grids;  // device
-  BatchItem* items;        // device, one per tile (mode 1 only)
   int ngrids;
   int nitems;
   int tile_x, tile_y;
   int ksteps;
   int64_t nsteps;
-  unsigned int* barrier;   // device counter, zeroed before each launch
-  unsigned long long* claim;  // device tile-claim counter, zeroed before each launch
+  unsigned int* barrier;   // device counter (mode 0), zeroed by each call
   int* err;
   unsigned long long wait_ns;  // limit of each barrier wait
   int skip_block;              // test hook: this block skips its first arrival (-1: none)
-  int mode;                    // 0: trapezoid tiles (k sweeps per pass); 1: two-sweep
-                               // register tiles (64 x 64, two sweeps per pass)
+  int mode;                    // 0: trapezoid tiles (k sweeps per pass); 1: register strips
+  // mode 1, per depth (strip_depth_index):
+  const int* first;            // device, [kStripDepths][ngrids + 1]: first unit of each grid
+  int units[kStripDepths];     // units of a pass
+  int chunk[kStripDepths];     // rows per unit
+  int64_t passes;
 };
+// pinned: the grid list and (mode 1) the unit lists as they go into the
+// workspace from p.grids on, `bytes` long (a multiple of 16).
 cudaError_t launch_batch(const BatchPlanDev& p, const StencilDesc& s, int dtype, int blocks,
-                         cudaStream_t st);
+                         const void* pinned, size_t bytes, cudaStream_t st);
 int batch_max_blocks(const StencilDesc& s, int dtype, int tile_x, int tile_y, int ksteps,
                      int mode = 0);
-// Tile of the two-sweep batched tiles (mode 1).
-constexpr int kBatchTb2X = 64, kBatchTb2Y = 64;
+int batch_strip_valid(int radius, int k);
+// The batch workspace is sized by 64 bytes per 64 x 64 tile.
+constexpr int kBatchTileX = 64, kBatchTileY = 64;
 size_t trap_smem_bytes(int dtype, int nf, int tile_x, int tile_y, int halo, int stages = 1);
 
 void count_launches(int64_t n);

@@ -174,7 +174,7 @@ struct Strip {
     const int nx = g.nx, ny = g.ny;
     const int x = x0 + (lane - G::HL) * V;  // this lane's first column
     const int yb = y0 - K * R;              // row of step 0
-    const int rows = y1 - y0, nsteps = rows + 2 * K * R;
+    const int nsteps = (y1 - y0) + 2 * K * R;
     // Source columns, wrapped (a column past a Dirichlet side stages a cell of
     // the row, which the mask replaces).
     int gx[VEC ? 1 : V];
@@ -210,12 +210,15 @@ struct Strip {
     };
 
     const uint32_t rbase = smem_u32(ring);
-    int lw = wrap(yb, ny);                            // row of the next copy
-    int64_t lrow = int64_t(lw) * nx + (VEC ? gx[0] : 0);  // its element offset
+    int lw = wrap(yb, ny);  // row of the next copy
+    // One field: a running source pointer; several: the kernel's pointers (in
+    // constant memory) plus one running offset.
+    int64_t lrow = int64_t(lw) * nx + (VEC ? gx[0] : 0);
+    const T* src = in[0] + lrow;
     auto copy_row = [&](uint32_t slot) {
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
-        const T* row = in[f] + lrow;
+        const T* row = NF == 1 ? src : in[f] + lrow;
         const uint32_t d = rbase + f * RING + slot;
         if constexpr (VEC) {
           cp_async_vec<VB>(d + lane * VB, row);
@@ -225,11 +228,15 @@ struct Strip {
             cp_async_elem<int(sizeof(T))>(d + (lane + 32 * j) * int(sizeof(T)), row + gx[j]);
         }
       }
-      lrow += nx;
-      if (++lw == ny) {
-        lw = 0;
-        lrow -= int64_t(ny) * nx;
+      const bool end = ++lw == ny;
+      if constexpr (NF == 1) {
+        src += nx;
+        if (end) src -= int64_t(ny) * nx;
+      } else {
+        lrow += nx;
+        if (end) lrow -= int64_t(ny) * nx;
       }
+      if (end) lw = 0;
     };
     if constexpr (!VEC) __syncwarp();
 #pragma unroll 1
@@ -241,6 +248,7 @@ struct Strip {
     C q[K][NQ][NF][V];
     const int nv = lane < G::HL || lane >= 32 - G::HL ? 0 : max(0, min(V, nx - x));
     int64_t orow = int64_t(y0 - 2 * K * R) * nx + x;  // output offset of step t's stored row
+    T* dst = out[0] + orow;
     uint32_t rd = 0;                                  // ring slot of row t
     auto step = [&](auto ph_tag, int t) {
       constexpr int PH = decltype(ph_tag)::value;  // t mod NQ
@@ -291,13 +299,14 @@ struct Strip {
           }
         }
         if constexpr (L == K) {
-          if (unsigned(t - 2 * K * R) < unsigned(rows)) {
+          if (t >= 2 * K * R && t < nsteps) {
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
+              T* d = NF == 1 ? dst : out[f] + orow;
               if constexpr (VEC) {
-                if (nv > 0) strip_store(out[f] + orow, o[f]);
+                if (nv > 0) strip_store(d, o[f]);
               } else {
-                strip_store_n(out[f] + orow, o[f], nv);
+                strip_store_n(d, o[f], nv);
               }
             }
           }
@@ -319,7 +328,8 @@ struct Strip {
       if constexpr (K >= 6) level(StripTag<6>());
       if constexpr (K >= 7) level(StripTag<7>());
       if constexpr (K >= 8) level(StripTag<8>());
-      orow += nx;
+      if constexpr (NF == 1) dst += nx;
+      else orow += nx;
       rd = (rd + ROWB) & (RING - 1);
     };
     // The step count is rounded up to the queue's period: the rows of the

@@ -156,3 +156,35 @@ def test_strips_write_only_their_output(lope, shape):
         for b in bufs:
             assert bool((b[:guard] == sentinel).all()) and bool((b[guard + n:] == sentinel).all())
         assert torch.equal(u, keep)
+
+
+@pytest.mark.parametrize("kind,prm,halo,depths", [("jacobi5", [0.2], 1, (8, 4, 2, 1)),
+                                                  ("star9r2", [0.1], 2, (4, 2, 1))])
+def test_batched_strips_equal_each_grid_alone(lope, kind, prm, halo, depths):
+    """Uneven grids of aligned and odd widths (fewer columns than a lane's,
+    one strip, several), both boundary kinds, every depth and a sweep count
+    that takes passes of each; then again in memory freed and allocated anew."""
+    shapes = [(1, 7), (130, 3), (40, 4), (65, 113), (200, 224), (17, 500), (300, 251), (90, 120)]
+    st = lope.Stencil.builtin(kind, *prm)
+
+    def once(T, launch):
+        grids, ins = [], []
+        for i, s in enumerate(shapes):
+            g = lope.Grid(s, "f32", halo=halo)
+            if i % 2 == 0:
+                g.set_boundaries([(1, 1), (1, 1)], [(0.3, -0.2), (0.0, 0.5)])
+            grids.append(g)
+            ins.append(to_device(LI.uniform_field(1850 + i, s), "f32")[0])
+        outs = lope.apply_batch(grids, st, ins, nsteps=T, launch=launch)
+        torch.cuda.synchronize()
+        lope.sync_status()
+        for g, u, o in zip(grids, ins, outs):
+            ref = lope.apply(g, st, u, nsteps=T, launch=lope.Launch(DIRECT, 0, 0, 0, -1))
+            assert torch.equal(ref, o), (g.shape, T)
+
+    for k in depths:
+        once(k, lope.Launch(STRIP, 0, 0, k, -1))
+        once(2 * k + 1, lope.Launch(STRIP, 0, 0, k, -1))
+    for _ in range(2):
+        once(15, None)
+        torch.cuda.empty_cache()
