@@ -21,7 +21,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "liblope.so")
 SOURCES = ["k_tma.cu", "k_tma_stage.cu", "k_generic.cu", "k_generic_rk.cu", "k_batch.cu",
-           "k_reduce.cu", "k_strip_diff.cu", "k_strip_swe.cu", "k_strip_linear.cu", "jit.cu", "api.cu"]
+           "k_reduce.cu", "k_strip_diff.cu", "k_strip_swe.cu", "k_strip_linear.cu", "k_brick.cu", "jit.cu", "api.cu"]
 # Device headers embedded in the library for run-time compiled local functions
 # (jit.cu hands them to NVRTC); they compile under nvcc and NVRTC alike.
 JIT_HEADERS = ["lope_internal.h", "device_common.cuh", "tma_device.cuh", "trap.cuh",

@@ -232,11 +232,26 @@ int64_t count_passes(const Choice& c, int64_t nsteps) {
 // query or log the plan of a short call see the path they always saw.
 constexpr int64_t kStripSteps = 12;
 
-// The strip choice for a grid, if the strips take it (they measured faster than
-// every other path there).
+// The strip choice for a grid: where the strips (2D) or bricks (3D) take it and
+// measured faster than the other paths.
 bool strip_choice(StepArgs a, Choice* c) {
   a.ksteps = a.s.stages >= 2 ? 1 : strip_kmax_of(a);
   if (!strip_supported(a)) return false;
+  if (a.g.ndim == 3) {
+    // Rows TMA cannot stage always gain (diff7 FP32, us per sweep: 100 x 333 x 77
+    // 26.4 -> 6.8, 130 x 500 x 510 75.8 -> 34.1, 511^3 278 -> 105).  On rows it can,
+    // the z-marches hold the small grids (128^3 5.5 / 5.3 us, 64^3 3.1 / 4.9), short
+    // ones (a chunk's fill is 8 planes: 16 x 256 x 256 4.0 / 5.3) and those whose
+    // blocks would be mostly halo; from 2^22 points on the bricks do better (64 x
+    // 128 x 512 7.5 -> 5.9, 256^3 periodic 26.0 -> 13.5, 512^3 110 -> 73.6, BF16
+    // 512^3 123 -> 70.6).
+    StepArgs one = a;
+    one.ksteps = 1;
+    const Geom& g = a.g;
+    if (tma_supported(one) && (npts(g) < (int64_t(1) << 22) || g.n[0] < 16 ||
+                               brick_cells(a) > 2 * g.n[1] * g.n[2]))
+      return false;
+  }
   *c = {kPathStrip, 0, 0, a.ksteps};
   return true;
 }
@@ -253,7 +268,7 @@ Choice default_choice(const Geom& g, const StencilDesc& s, const void* const* in
     if (it != g_tune.end() && choice_supported(a, it->second)) return it->second;
   }
   if (nsteps >= kStripSteps) {
-    // Register strips, FP32 / BF16.  Measured on GB300 against the choices
+    // Register strips and bricks, FP32 / BF16.  2D, measured on GB300 against the choices
     // below (which the same calls took before): jacobi5 FP32 7094^2 x20
     // (unaligned rows) 1.65 -> 0.38 ms, 100 x 200 x20 51 -> 39 us; star9r2 FP32
     // 8192^2 x50 3.03 -> 1.72 ms; linear shallow water 4096^2 x3 x200 FP32 7.86
@@ -456,6 +471,14 @@ cudaError_t issue_stages(const Geom& g, const StencilDesc& s, const Choice& c,
   return cudaSuccess;
 }
 
+// One sweep of a 3D grid: what the bricks (depths 4 and 2) leave of an odd
+// count, on the one-sweep kernel of the grid.
+cudaError_t launch_single(const StepArgs& a) {
+  if (tma_supported(a)) return launch_tma(a, nullptr);
+  if (march_supported(a)) return launch_march(a);
+  return launch_direct(a, nullptr);
+}
+
 // Issue the launch sequence: the passes of count_passes, ping-ponging between out
 // and work so that the last one writes out.
 cudaError_t issue(const Geom& g, const StencilDesc& s, const Choice& c, const void* const* in,
@@ -482,7 +505,7 @@ cudaError_t issue(const Geom& g, const StencilDesc& s, const Choice& c, const vo
       case kPathTma: e = launch_tma(a, nullptr); break;
       case kPathTrap: e = launch_trap2d(a); break;
       case kPathMarch: e = launch_march(a); break;
-      case kPathStrip: e = launch_strip(a); break;
+      case kPathStrip: e = a.ksteps == 1 && g.ndim == 3 ? launch_single(a) : launch_strip(a); break;
       default: e = launch_direct(a, nullptr); break;
     }
     if (e != cudaSuccess) return e;

@@ -1,0 +1,328 @@
+// Register bricks: K sweeps of a 3D radius-1 star function per pass, every
+// intermediate state in registers (device templates; compiles under nvcc and
+// NVRTC alike).  The 3D form of the register strips (strip_device.cuh).
+//
+// A block of WY half-warps owns a column of the grid, 64 columns (16 lanes of 4)
+// by WY x RY rows, and marches a chunk of planes along z.  At step t it takes plane
+// t of the input and computes plane t-l of every level l = 1 .. K (the state
+// after l sweeps) from the last three planes of level l-1 in registers; level K
+// is stored.  Taps along z come from that queue, along x from the lane's own
+// columns and by shuffle from its neighbours, along y from the thread's own
+// rows and, past them, from the first and last rows of the neighbouring
+// half-warps, which each leaves in shared memory once per plane and level.  All
+// levels of a step read rows that were left one step before, so one block
+// barrier per plane is enough.  The outer K rows and 4 columns of the column
+// are computed again by the neighbouring blocks.  Planes arrive in a private
+// ring of shared memory per warp through cp.async, PF planes ahead, from
+// source rows and columns fixed for the whole march (periodic sides already
+// wrapped).
+//
+// Dirichlet sides: the first and last column of blocks start and end at the
+// grid's side, so the values past it are what the outermost lanes see instead
+// of a shuffle and the outermost half-warps instead of an exchanged row; neither
+// needs a mask in the steady loop (masking the cells past a side level by level
+// cost 1.6x at 512^3).  Only the planes past a z side are set, in loops of their
+// own over the first and last steps.  Each level is rounded to the storage
+// precision: bitwise the result of K one-sweep launches.
+//
+// What bounds it: instruction issue and its latencies, with 8 warps per SM.
+// One block of 16 half-warps x 4 rows and up to 255 registers measured best
+// (diff7 FP32, us per sweep, 512^3 Dirichlet / 256^3 periodic / 130 x 500 x 510):
+//   K = 4: 73.5 / 13.4 / 33.9 (244 registers)
+//   K = 3: 77.2 / 15.1 / 37.3 (197); 12 half-warps, two blocks of 168: 95 / 18 / 51
+//   K = 2: 95.5 / 17.5 / 52; 5 or 6 rows per thread were no better
+// against 109 (two sweeps per launch) / 25.4 / 75.7 (one) on the z-marches.  Tiles
+// 64 columns wide waste less of a 256- or 512-wide grid than 128 (a warp per
+// row): 1.97 -> 1.41 times the points at 256^3.
+#pragma once
+
+#include "strip_device.cuh"
+
+namespace lope {
+
+namespace {
+
+__device__ __forceinline__ void brick_store_n(float* d, const float (&w)[4], int j0, int j1) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (i >= j0 && i < j1) d[i] = w[i];
+}
+
+// Taps of column p of row r of a level: center plane c (rows of this thread),
+// the rows beyond them, the columns beyond the lane's, the planes below and above.
+template <int RY>
+struct BrickAcc {
+  const float (&c)[RY][kStripV];
+  const float (&zm)[RY][kStripV];
+  const float (&zp)[RY][kStripV];
+  const float (&up)[kStripV];  // row -1
+  const float (&dn)[kStripV];  // row RY
+  float xl, xr;                // columns -1 and V of row r
+  int r, p;
+  __device__ __forceinline__ float operator()(int, int dx, int dy, int dz) const {
+    if (dz != 0) return dz < 0 ? zm[r][p] : zp[r][p];
+    if (dy != 0) return r + dy < 0 ? up[p] : r + dy >= RY ? dn[p] : c[r + dy][p];
+    return p + dx < 0 ? xl : p + dx >= kStripV ? xr : c[r][p + dx];
+  }
+  __device__ __forceinline__ int64_t gidx() const { return 0; }
+};
+
+}  // namespace
+
+struct BrickGrid {
+  int nx, ny, nz;
+  int bc[3][2];        // z, y, x
+  float bval[3][2];
+};
+
+template <class Op, class T> struct BrickParams {
+  Op op;
+  const T* in;
+  T* out;
+  BrickGrid g;
+  int tiles_x, tiles_y, zchunk;
+};
+
+template <class T, int K, int RY, int WY> struct BrickGeom {
+  static constexpr int LX = 16;                            // lanes along x
+  static constexpr int HL = 1;                             // halo lanes per side (K <= 4 columns)
+  static constexpr int BX = LX * kStripV, BY = WY * RY;    // cells of a block
+  static constexpr int THREADS = WY * LX;
+  static constexpr int ROWB = LX * kStripV * int(sizeof(T));
+  static constexpr int D = 4;                              // ring planes
+  static constexpr int RING = D * RY * ROWB;               // bytes per half-warp
+  static constexpr int EXROW = LX * kStripV * 4;           // an exchanged row (FP32)
+  static constexpr int EXL = (WY + 2) * 2 * EXROW;         // a level's rows: half-warps -1 .. WY
+  static constexpr int EX = K * EXL;                       // one of two exchange buffers
+  static constexpr int SMEM = WY * RING + 2 * EX;
+};
+
+// Block i of n along an axis of extent m, blocks of b cells whose outer h are
+// halo: first cell c and outputs [o0, o1).  A Dirichlet side needs no halo: the
+// first block then starts at cell 0, the last ends at cell m - 1 (m >= b).
+struct BrickSpan { int c, o0, o1; };
+__host__ __device__ inline BrickSpan brick_span(int i, int n, int m, int b, int h, bool dlo, bool dhi) {
+  const int v = b - 2 * h;
+  BrickSpan s;
+  s.c = i * v - (dlo ? 0 : h);
+  s.o0 = i == 0 ? 0 : s.c + h;
+  s.o1 = s.c + b - h < m ? s.c + b - h : m;
+  if (dhi && i == n - 1) {
+    s.c = m - b;
+    s.o1 = m;
+  }
+  return s;
+}
+__host__ __device__ inline int brick_count(int m, int b, int h, bool dlo, bool dhi) {
+  const int v = b - 2 * h, r = m - (dlo ? h : 0) - (dhi ? h : 0);
+  return r <= v ? 1 : (r + v - 1) / v;
+}
+
+namespace {
+
+template <class Op, class T, int K, int RY, int WY, bool VEC>
+struct Brick {
+  using G = BrickGeom<T, K, RY, WY>;
+  static_assert(Op::R == 1 && Op::NF == 1 && Op::STAR && K <= 4, "radius-1 star function of one field");
+  static constexpr int V = kStripV, VB = V * int(sizeof(T)), D = G::D, PF = D - 1;
+
+  static __device__ __forceinline__ void march(const BrickParams<Op, T>& p, unsigned char* smem,
+                                               const BrickSpan& sx, const BrickSpan& sy, int z0, int z1) {
+    const BrickGrid& g = p.g;
+    const int lane = threadIdx.x % G::LX, wy = threadIdx.x / G::LX;
+    const int nx = g.nx, ny = g.ny, nz = g.nz;
+    const int x = sx.c + lane * V;
+    const int yw = sy.c + wy * RY;  // first row of this half-warp
+    const int nsteps = (z1 - z0) + 2 * K;
+    int gx[VEC ? 1 : V];
+    if constexpr (VEC) {
+      gx[0] = wrap(x, nx);
+    } else {
+#pragma unroll
+      for (int j = 0; j < V; ++j) gx[j] = wrap(sx.c + lane + G::LX * j, nx);
+    }
+    int roff[RY];  // source rows, wrapped
+#pragma unroll
+    for (int r = 0; r < RY; ++r) roff[r] = wrap(yw + r, ny) * nx + (VEC ? gx[0] : 0);
+    // What the outermost lanes see past their columns: the value of the
+    // Dirichlet side the block ends at (elsewhere they are halo lanes, whose
+    // results nothing reads).
+    const float vxl = g.bval[2][0], vxr = g.bval[2][1];
+    const bool first = lane == 0, last = lane == G::LX - 1;
+    constexpr int kFar = 1 << 30;
+    const int zlo = g.bc[0][0] == kDirichlet ? 0 : -kFar, zhi = g.bc[0][1] == kDirichlet ? nz : kFar;
+
+    unsigned char* ring = smem + wy * G::RING;
+    const uint32_t rbase = smem_u32(ring);
+    // Exchanged rows (two buffers, used in turn): per level and half-warp its
+    // first and last row.  Own rows, and the neighbours' rows beside them.
+    // The rows of half-warps -1 and WY hold the Dirichlet y sides' values.
+    constexpr int EXR = G::EXROW / 4, EXL = G::EXL / 4;  // floats per row, per level
+    float* ex = reinterpret_cast<float*>(smem + WY * G::RING) + 2 * EXR + lane * V;
+    for (int i = threadIdx.x; i < 2 * K * 2 * EXR; i += G::THREADS) {
+      const int lv = i / (2 * EXR), j = i % (2 * EXR);  // buffer and level, row and column
+      float* e = reinterpret_cast<float*>(smem + WY * G::RING) + lv * EXL;
+      if (j < EXR) e[EXR + j] = g.bval[1][0];
+      else e[(WY + 1) * 2 * EXR + j - EXR] = g.bval[1][1];
+    }
+    float* exw = ex + wy * 2 * EXR;
+    const float* exu = exw - EXR;
+    const float* exd = exw + 2 * EXR;
+    const int64_t plane = int64_t(nx) * ny;
+    int lz = wrap(z0 - K, nz);
+    const T* src = p.in + int64_t(lz) * plane;
+    auto copy_plane = [&](uint32_t slot) {
+#pragma unroll
+      for (int r = 0; r < RY; ++r) {
+        const uint32_t d = rbase + slot + r * (D * G::ROWB);
+        const T* row = src + roff[r];
+        if constexpr (VEC) {
+          cp_async_vec<VB>(d + lane * VB, row);
+        } else {
+#pragma unroll
+          for (int j = 0; j < V; ++j)
+            cp_async_elem<int(sizeof(T))>(d + (lane + G::LX * j) * int(sizeof(T)), row + gx[j]);
+        }
+      }
+      src += plane;
+      if (++lz == nz) {
+        lz = 0;
+        src -= int64_t(nz) * plane;
+      }
+    };
+#pragma unroll 1
+    for (int t = 0; t < PF; ++t) {
+      if (t < nsteps) copy_plane(t * G::ROWB);
+      cp_async_commit();
+    }
+
+    float q[K][3][RY][V];
+    // output columns [jv0, jv1) of this lane (aligned rows: all or none)
+    const int jv0 = max(0, sx.o0 - x), jv1 = min(V, sx.o1 - x);
+    T* dst = p.out + (int64_t(z0 - 2 * K) * ny + yw) * nx + x;  // row 0 of step t's stored plane
+    uint32_t rd = 0;
+    // bit r: row r is an output row of this lane
+    unsigned ok = 0;
+#pragma unroll
+    for (int r = 0; r < RY; ++r) {
+      if (jv0 < jv1 && yw + r >= sy.o0 && yw + r < sy.o1) ok |= 1u << r;
+    }
+    auto put_row = [&](float* d, const float (&w)[V]) {
+      *reinterpret_cast<float4*>(d) = make_float4(w[0], w[1], w[2], w[3]);
+    };
+    __syncthreads();
+    auto step = [&](auto ph_tag, auto z_tag, int t) {
+      constexpr bool ZEDGE = decltype(z_tag)::value != 0;  // levels may lie past a z side
+      // a level's plane past a Dirichlet z side holds its value
+      auto mask = [&](float (&w)[RY][V], int z) {
+        if (z < zlo || z >= zhi) {
+#pragma unroll
+          for (int r = 0; r < RY; ++r)
+#pragma unroll
+            for (int j = 0; j < V; ++j) w[r][j] = z < zlo ? g.bval[0][0] : g.bval[0][1];
+        }
+      };
+      constexpr int PH = decltype(ph_tag)::value;  // t mod 3
+      const int nb = (t & 1) * (G::EX / 4), ob = G::EX / 4 - nb;
+      float* const wrow = exw + nb;
+      const float* const urow = exu + ob;
+      const float* const drow = exd + ob;
+      cp_async_wait<PF - 1>();
+      if constexpr (!VEC) __syncwarp();
+#pragma unroll
+      for (int r = 0; r < RY; ++r)
+        strip_load(reinterpret_cast<const T*>(ring + rd + r * (D * G::ROWB)) + lane * V, q[0][PH][r]);
+      if constexpr (!VEC) __syncwarp();
+      if (t + PF < nsteps) copy_plane((rd + PF * G::ROWB) & (D * G::ROWB - 1));
+      cp_async_commit();
+      if constexpr (ZEDGE) mask(q[0][PH], z0 - K + t);
+      put_row(wrow, q[0][PH][0]);
+      put_row(wrow + EXR, q[0][PH][RY - 1]);
+      auto level = [&](auto l_tag) {
+        constexpr int L = decltype(l_tag)::value;
+        // slots of level L-1: newest plane, the center one before it, the one below
+        constexpr int ZP = ((PH - (L - 1)) % 3 + 3) % 3, CC = (ZP + 2) % 3, ZM = (ZP + 1) % 3;
+        float up[V], dn[V];
+        strip_load(urow + (L - 1) * EXL, up);
+        strip_load(drow + (L - 1) * EXL, dn);
+        float o[RY][V];
+#pragma unroll
+        for (int r = 0; r < RY; ++r) {
+          float xl = shfl_left(q[L - 1][CC][r][V - 1]), xr = shfl_right(q[L - 1][CC][r][0]);
+          if (first) xl = vxl;
+          if (last) xr = vxr;
+#pragma unroll
+          for (int j = 0; j < V; ++j) {
+            BrickAcc<RY> acc{q[L - 1][CC], q[L - 1][ZM], q[L - 1][ZP], up, dn, xl, xr, r, j};
+            float res[1], unused = 0.f;
+            p.op(acc, res, unused);
+            o[r][j] = res[0];
+          }
+        }
+        if constexpr (L == K) {
+          if (t >= 2 * K && t < nsteps) {
+#pragma unroll
+            for (int r = 0; r < RY; ++r)
+              if (ok >> r & 1) {
+                if constexpr (VEC) strip_store(dst + int64_t(r) * nx, o[r]);
+                else brick_store_n(dst + int64_t(r) * nx, o[r], jv0, jv1);
+              }
+          }
+        } else {
+          constexpr int W = ((PH - L) % 3 + 3) % 3;  // slot of plane t - L
+#pragma unroll
+          for (int r = 0; r < RY; ++r) strip_round<T>(o[r]);
+          if constexpr (ZEDGE) mask(o, z0 - K + t - L);
+#pragma unroll
+          for (int r = 0; r < RY; ++r)
+#pragma unroll
+            for (int j = 0; j < V; ++j) q[L][W][r][j] = o[r][j];
+          put_row(wrow + L * EXL, o[0]);
+          put_row(wrow + L * EXL + EXR, o[RY - 1]);
+        }
+      };
+      level(StripTag<1>());
+      if constexpr (K >= 2) level(StripTag<2>());
+      if constexpr (K >= 3) level(StripTag<3>());
+      if constexpr (K >= 4) level(StripTag<4>());
+      dst += plane;
+      rd = (rd + G::ROWB) & (D * G::ROWB - 1);
+      __syncthreads();
+    };
+    // Steps run in threes (the queue's period); planes whose level is not
+    // complete yet, and those past z1, are computed and dropped.
+    int t = 0;
+    auto run_to = [&](auto z_tag, int end) {
+#pragma unroll 1
+      for (; t < end; t += 3) {
+        step(StripTag<0>(), z_tag, t);
+        step(StripTag<1>(), z_tag, t + 1);
+        step(StripTag<2>(), z_tag, t + 2);
+      }
+    };
+    run_to(StripTag<1>(), z0 - K < zlo ? 2 * K : 0);
+    run_to(StripTag<0>(), z1 + K > zhi ? nsteps - 2 * K - 2 : nsteps);
+    run_to(StripTag<1>(), nsteps);
+    cp_async_wait<0>();
+  }
+};
+
+template <class Op, class T, int K, int RY, int WY, int MINB, bool VEC>
+__global__ void __launch_bounds__(BrickGeom<T, K, RY, WY>::THREADS, MINB) brick3d_kernel(const __grid_constant__ BrickParams<Op, T> p) {
+  using B = Brick<Op, T, K, RY, WY, VEC>;
+  using G = typename B::G;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int ntiles = p.tiles_x * p.tiles_y;
+  const int tile = blockIdx.x % ntiles, zc = blockIdx.x / ntiles;
+  const int z0 = zc * p.zchunk, z1 = min(p.g.nz, z0 + p.zchunk);
+  if (z0 >= z1) return;
+  const BrickGrid& g = p.g;
+  const BrickSpan sx = brick_span(tile % p.tiles_x, p.tiles_x, g.nx, G::BX, G::HL * kStripV,
+                                  g.bc[2][0] == kDirichlet, g.bc[2][1] == kDirichlet);
+  const BrickSpan sy = brick_span(tile / p.tiles_x, p.tiles_y, g.ny, G::BY, K,
+                                  g.bc[1][0] == kDirichlet, g.bc[1][1] == kDirichlet);
+  B::march(p, smem_raw, sx, sy, z0, z1);
+}
+
+}  // namespace
+}  // namespace lope

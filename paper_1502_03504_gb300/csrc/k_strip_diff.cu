@@ -5,12 +5,14 @@
 namespace lope {
 
 int strip_kmax_of(const StepArgs& a) {
+  if (a.g.ndim == 3) return kBrickK;
   if (a.s.kind == kUser) return kStripUserK;
   return strip_kmax(a.g.nf, a.s.radius, a.s.star);
 }
 
 bool strip_supported(const StepArgs& a) {
   const Geom& g = a.g;
+  if (g.ndim == 3) return brick_supported(a);
   if (g.ndim != 2 || a.adjoint || a.stage >= 2 || g.dtype == kF64 || has_external(g)) return false;
   if (a.s.radius < 1 || a.s.radius > 2 || g.n[1] > (int64_t(1) << 30) || g.n[2] > (int64_t(1) << 30))
     return false;
@@ -27,6 +29,7 @@ bool strip_supported(const StepArgs& a) {
 }
 
 cudaError_t launch_strip(const StepArgs& a) {
+  if (a.g.ndim == 3) return launch_brick(a);
   switch (a.s.kind) {
     case kUser: return jit_launch(a, kPathStrip);
     case kJacobi5: return strip_op(a, OpJacobi5{a.s.prm[0]});

@@ -118,6 +118,11 @@ cudaError_t launch_strip(const StepArgs& a);
 cudaError_t launch_strip_swe(const StepArgs& a);
 cudaError_t launch_strip_linear(const StepArgs& a);
 bool strip_supported(const StepArgs& a);
+// Register bricks (brick_device.cuh), the 3D form of path 5.
+cudaError_t launch_brick(const StepArgs& a);
+bool brick_supported(const StepArgs& a);
+int64_t brick_cells(const StepArgs& a);  // cells of the blocks that cover a plane, halo included
+constexpr int kBrickK = 4;
 int strip_kmax_of(const StepArgs& a);
 constexpr int kStripUserK = 4;  // depth of run-time compiled functions
 // Run-time compiled local functions (jit.cu).

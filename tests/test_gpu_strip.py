@@ -188,3 +188,51 @@ def test_batched_strips_equal_each_grid_alone(lope, kind, prm, halo, depths):
     for _ in range(2):
         once(15, None)
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("shape", [(3, 64, 64), (9, 65, 68), (20, 120, 120), (50, 177, 236), (33, 64, 612)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_bricks_bitwise_equal_direct(lope, shape, dtype):
+    """The 3D form: one to several blocks per axis, chunks shorter and longer
+    than the pipeline, each axis periodic or Dirichlet with zero and non-zero
+    values, sweep counts that end on depths 4, 2 and 1."""
+    st = lope.Stencil.builtin("diff7", 0.1)
+    u, _ = to_device(LI.uniform_field(1860, shape), dtype)
+    for bcs in ([0, 0, 0], [1, 1, 1], [1, 0, 1], [0, 1, 0], [0, 0, 1]):
+        for bv in (None, [(0.3, -0.2), (0.1, 0.5), (-0.4, 0.7)]):
+            g = lope.Grid(shape, dtype, halo=1).set_boundaries(bcs, bv)
+            for T, k in ((4, 4), (2, 2), (7, 4), (3, 2)):
+                _check(lope, g, st, [u], T, k)
+
+
+@pytest.mark.parametrize("shape", [(5, 64, 65), (20, 121, 127), (31, 70, 301)], ids=lambda s: "x".join(map(str, s)))
+def test_bricks_rows_of_any_pitch_and_tables(lope, shape):
+    rng = np.random.default_rng(1861)
+    w = np.zeros((3, 3, 3))
+    for i in ((0, 1, 1), (2, 1, 1), (1, 0, 1), (1, 2, 1), (1, 1, 0), (1, 1, 2)):
+        w[i] = rng.uniform(0.02, 0.12)
+    w[1, 1, 1] = 1.0 - w.sum()
+    u, _ = to_device(LI.uniform_field(1862, shape), "f32")
+    for st in (lope.Stencil.builtin("diff7", 0.1), lope.Stencil.linear(w)):
+        for bcs in ([0, 0, 0], [1, 1, 1], [1, 0, 1], [0, 1, 0]):
+            g = lope.Grid(shape, "f32", halo=1).set_boundaries(bcs, [0.5 if b else 0.0 for b in bcs])
+            _check(lope, g, st, [u], 9, 4)
+
+
+def test_bricks_write_only_their_output(lope):
+    shape = (21, 70, 133)
+    n = int(np.prod(shape))
+    guard, sentinel = 4096, -7.0e30
+    u = torch.rand(shape, device="cuda")
+    keep = u.clone()
+    st = lope.Stencil.builtin("diff7", 0.1)
+    for bc in ([0, 0, 0], [1, 1, 1]):
+        g = lope.Grid(shape, "f32", halo=1).set_boundaries(bc)
+        bufs = [torch.full((n + 2 * guard,), sentinel, device="cuda") for _ in range(2)]
+        out, work = (b[guard:guard + n].view(shape) for b in bufs)
+        lope.apply(g, st, u, out=out, work=work, nsteps=10, launch=lope.Launch(STRIP, 0, 0, 4, -1))
+        torch.cuda.synchronize()
+        for b in bufs:
+            assert bool((b[:guard] == sentinel).all()) and bool((b[guard + n:] == sentinel).all())
+        assert torch.equal(u, keep)
