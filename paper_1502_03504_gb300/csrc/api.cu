@@ -702,6 +702,12 @@ lope_status forward_ckpt_impl(const lope_grid* grid, const lope_stencil* st, con
                               cudaStream_t stream) {
   void* tmp = ws + L.off_tmp;
   const void* cur = u0;
+  // A segment's sweeps take the strips / bricks from half their planner's count
+  // on: the segments follow one another, so their fill is paid once per depth.
+  StepArgs probe = base_args(grid->g, st->s, nullptr, nullptr);
+  probe.in[0] = u0;
+  Choice sc;
+  const bool strips = K >= kStripSteps / 2 && strip_choice(probe, &sc);
   for (int64_t i = 0; i < L.nseg; ++i) {
     const int64_t len = std::min<int64_t>(K, nsteps - i * K);
     void* dst = (i == L.nseg - 1) ? uT : static_cast<void*>(ws + L.off_ckpt + size_t(i) * L.field);
@@ -709,6 +715,10 @@ lope_status forward_ckpt_impl(const lope_grid* grid, const lope_stencil* st, con
     void* out1[1] = {dst};
     void* work1[1] = {tmp};
     lope_launch cfg = {0, 0, 0, 0, -1};
+    if (strips) {
+      cfg.path = kPathStrip;
+      cfg.tsteps = sc.k;
+    }
     lope_status rs = apply_impl(grid, st, in1, out1, work1, len, &cfg, stream);
     if (rs != LOPE_OK) return rs;
     cur = dst;
@@ -739,12 +749,20 @@ lope_status reverse_impl(const lope_grid* grid, const lope_stencil* st, const vo
   const bool diffusion = s.kind != kLinear;
   const StencilDesc sa = diffusion ? s : reflected(s);
   double* partials = reinterpret_cast<double*>(ws + L.off_part);
-  cudaError_t e = cudaMemsetAsync(partials, 0, sizeof(double) * L.partials, stream);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+  cudaError_t e = launch_zero(partials, L.partials, stream);
+  if (e != cudaSuccess) return cuda_fail(e, "zeroing the partial sums");
   StepArgs probe = base_args(ga, sa, err, stream);
   probe.in[0] = lamT;
   probe.adjoint = diffusion;
   const bool tma = tma_supported(probe);
+  // 3D diffusion on grids the planner gives the bricks: recompute four states
+  // and run two adjoint steps per pass.
+  Choice sc;
+  probe.in[0] = u0;
+  probe.adjoint = false;
+  probe.g = g;
+  const bool brick = diffusion && g.ndim == 3 && aligned16(u0) && brick_adjoint_supported(probe) && strip_choice(probe, &sc);
+  int turn = 0;  // lambda buffers used in turn
   int blocks_used = 0;
   const void* lam = lamT;
   int64_t m = 0;  // adjoint steps done
@@ -753,8 +771,21 @@ lope_status reverse_impl(const lope_grid* grid, const lope_stencil* st, const vo
     const void* ck = i == 0 ? u0 : static_cast<const void*>(ws + L.off_ckpt + size_t(i - 1) * L.field);
     // recompute u_{s0+1} .. u_{s0+len-1}
     const void* prev = ck;
-    for (int64_t j = 1; j < len; ++j) {
-      void* dst = ws + L.off_seg + size_t(j - 1) * L.field;
+    auto seg = [&](int64_t j) { return static_cast<void*>(ws + L.off_seg + size_t(j - 1) * L.field); };
+    int64_t j1 = 1;
+    while (brick && len - j1 >= 2) {  // states j1 .. j1 + k - 1
+      const int k = len - j1 >= 4 ? 4 : 2;
+      StepArgs a = base_args(g, s, err, stream);
+      a.in[0] = prev;
+      a.ksteps = k;
+      void* outs[4] = {nullptr, nullptr, nullptr, nullptr};
+      for (int l = 0; l < k; ++l) outs[l] = seg(j1 + l);
+      if ((e = launch_brick_states(a, outs)) != cudaSuccess) return cuda_fail(e, "recomputing states");
+      j1 += k;
+      prev = seg(j1 - 1);
+    }
+    for (int64_t j = j1; j < len; ++j) {
+      void* dst = seg(j);
       const void* in1[1] = {prev};
       void* out1[1] = {dst};
       lope_launch cfg = {0, 0, 0, 0, -1};
@@ -762,19 +793,28 @@ lope_status reverse_impl(const lope_grid* grid, const lope_stencil* st, const vo
       if (rs != LOPE_OK) return rs;
       prev = dst;
     }
-    for (int64_t j = len - 1; j >= 0; --j, ++m) {
-      const void* ut = j == 0 ? ck : static_cast<const void*>(ws + L.off_seg + size_t(j - 1) * L.field);
-      void* dst = (m == nsteps - 1) ? grad_u0
-                                    : static_cast<void*>(ws + L.off_lam + size_t(m & 1) * L.field);
+    auto state = [&](int64_t j) { return j == 0 ? ck : static_cast<const void*>(seg(j)); };
+    for (int64_t j = len - 1; j >= 0;) {
+      const int k = brick && j >= 1 ? 2 : 1;
+      m += k;
+      void* dst = m == nsteps ? grad_u0 : static_cast<void*>(ws + L.off_lam + size_t(turn) * L.field);
+      turn ^= 1;
       StepArgs a = base_args(ga, sa, err, stream);
       a.in[0] = lam;
       a.out[0] = dst;
-      a.adjoint = diffusion;
-      a.ut = ut;
       a.partials = partials;
       a.partial_count = L.partials;
       int b = 0;
-      e = tma ? launch_tma(a, &b) : launch_direct(a, &b);
+      if (k > 1) {
+        a.ksteps = k;
+        const void* uts[2] = {state(j), state(j - 1)};
+        e = launch_brick_adjoint(a, uts, &b);
+      } else {
+        a.adjoint = diffusion;
+        a.ut = state(j);
+        e = tma ? launch_tma(a, &b) : launch_direct(a, &b);
+      }
+      j -= k;
       if (e != cudaSuccess) return cuda_fail(e, "adjoint kernel launch");
       blocks_used = std::max(blocks_used, b);
       lam = dst;
@@ -784,7 +824,7 @@ lope_status reverse_impl(const lope_grid* grid, const lope_stencil* st, const vo
     if (diffusion) {
       e = launch_finalize(partials, std::max(blocks_used, 1), gc, 0, stream);
     } else {
-      e = cudaMemsetAsync(gc, 0, sizeof(double), stream);
+      e = launch_zero(gc, 1, stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, "finalize dL/dc");
   }

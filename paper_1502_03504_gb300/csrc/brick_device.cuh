@@ -75,10 +75,42 @@ struct BrickGrid {
   float bval[3][2];
 };
 
+// What a brick pass computes besides the state K sweeps on.
+enum : int {
+  kBrickPlain = 0,
+  kBrickStates = 1,  // every level's state is stored (a checkpoint segment's recomputation)
+  kBrickAdjoint = 2  // K steps of the transposed diffusion backward in time, each with its
+                     // sum of (L^T lambda) u_t over the grid (dL/dc)
+};
+// Both forms of the adjoint are near HBM's rate.  256^3 FP32, us per launch: four
+// states stored 75 (320 MB; four sweeps one at a time 98); two adjoint steps 61
+// (256 MB; one at a time 2 x 41).  The states u_t go to registers one step ahead
+// of their use: staged two planes deep in shared memory they took 67, three steps
+// per pass 104, and with the sums in FP64 (its pipe runs one warp instruction in
+// about 19 cycles) 77 and 114.
+
+// One step of lambda' = lambda + c L^T lambda; the second result is L^T lambda
+// (the operations of OpAdjDiffusion in the same order).
+struct OpBrickAdjoint {
+  static constexpr int R = 1, NF = 1;
+  static constexpr bool REDUCES = false, STAR = true;
+  Coef c;
+  template <class C, class A>
+  __device__ __forceinline__ void operator()(const A& U, C (&o)[1], C& lt) const {
+    const C l = U(0, 0, 0, 0);
+    const C nb = add(add(add(U(0, 1, 0, 0), U(0, -1, 0, 0)), add(U(0, 0, 1, 0), U(0, 0, -1, 0))),
+                     add(U(0, 0, 0, 1), U(0, 0, 0, -1)));
+    lt = fma_(C(-6), l, nb);
+    o[0] = fma_(c.get(C()), lt, l);
+  }
+};
+
 template <class Op, class T> struct BrickParams {
   Op op;
   const T* in;
-  T* out;
+  T* out[4];           // out[K-1]: the state K sweeps on; kBrickStates: out[l-1] level l
+  const T* ut[4];      // kBrickAdjoint: u_t of level l in ut[l-1]
+  double* partials;    // kBrickAdjoint: per-block sums, added to
   BrickGrid g;
   int tiles_x, tiles_y, zchunk;
 };
@@ -120,9 +152,10 @@ __host__ __device__ inline int brick_count(int m, int b, int h, bool dlo, bool d
 
 namespace {
 
-template <class Op, class T, int K, int RY, int WY, bool VEC>
+template <class Op, class T, int K, int RY, int WY, int MODE, bool VEC>
 struct Brick {
   using G = BrickGeom<T, K, RY, WY>;
+  static_assert(MODE == kBrickPlain || VEC, "the adjoint's forms stage whole vectors");
   static_assert(Op::R == 1 && Op::NF == 1 && Op::STAR && K <= 4, "radius-1 star function of one field");
   static constexpr int V = kStripV, VB = V * int(sizeof(T)), D = G::D, PF = D - 1;
 
@@ -171,6 +204,30 @@ struct Brick {
     const int64_t plane = int64_t(nx) * ny;
     int lz = wrap(z0 - K, nz);
     const T* src = p.in + int64_t(lz) * plane;
+    // output columns [jv0, jv1) of this lane (aligned rows: all or none)
+    const int jv0 = max(0, sx.o0 - x), jv1 = min(V, sx.o1 - x);
+    const int64_t rowoff = int64_t(yw) * nx + x;  // row 0 of this thread in a plane
+    T* dst = p.out[K - 1] + int64_t(z0 - 2 * K) * plane + rowoff;  // of step t's stored plane
+    uint32_t rd = 0;
+    // bit r: row r is an output row of this lane
+    unsigned ok = 0;
+#pragma unroll
+    for (int r = 0; r < RY; ++r) {
+      if (jv0 < jv1 && yw + r >= sy.o0 && yw + r < sy.o1) ok |= 1u << r;
+    }
+    // Planes of this pass's z range: out and ut hold plane z at z * plane.
+    int64_t zoff = int64_t(z0 - K) * plane;  // of step t's newest plane
+    // kBrickAdjoint: u_t of every level for the coming step, loaded to registers
+    // right after the level's last use of the step before.
+    float ut[MODE == kBrickAdjoint ? K : 1][RY][V];
+    auto load_state = [&](int l, int t) {  // the plane level l computes at step t, if in the chunk
+      if (unsigned(t - K - l) < unsigned(z1 - z0)) {
+        const T* s = p.ut[l - 1] + (int64_t(z0 - K + t - l) * plane);
+#pragma unroll
+        for (int r = 0; r < RY; ++r)
+          if (ok >> r & 1) strip_load(s + roff[r], ut[l - 1][r]);
+      }
+    };
     auto copy_plane = [&](uint32_t slot) {
 #pragma unroll
       for (int r = 0; r < RY; ++r) {
@@ -196,17 +253,8 @@ struct Brick {
       cp_async_commit();
     }
 
+    float sum = 0.f, low = 0.f;  // kBrickAdjoint: this thread's sum, and the rounding errors of it
     float q[K][3][RY][V];
-    // output columns [jv0, jv1) of this lane (aligned rows: all or none)
-    const int jv0 = max(0, sx.o0 - x), jv1 = min(V, sx.o1 - x);
-    T* dst = p.out + (int64_t(z0 - 2 * K) * ny + yw) * nx + x;  // row 0 of step t's stored plane
-    uint32_t rd = 0;
-    // bit r: row r is an output row of this lane
-    unsigned ok = 0;
-#pragma unroll
-    for (int r = 0; r < RY; ++r) {
-      if (jv0 < jv1 && yw + r >= sy.o0 && yw + r < sy.o1) ok |= 1u << r;
-    }
     auto put_row = [&](float* d, const float (&w)[V]) {
       *reinterpret_cast<float4*>(d) = make_float4(w[0], w[1], w[2], w[3]);
     };
@@ -246,17 +294,38 @@ struct Brick {
         strip_load(urow + (L - 1) * EXL, up);
         strip_load(drow + (L - 1) * EXL, dn);
         float o[RY][V];
+        // kBrickAdjoint: a chain of FMAs over a row's cells, added to the
+        // thread's sum with the addition's rounding error kept (two-sum), so
+        // the accumulation rounds like FP64 and leaves the slow FP64 pipe alone
+        const bool inside = MODE == kBrickAdjoint && unsigned(t - K - L) < unsigned(z1 - z0);
 #pragma unroll
         for (int r = 0; r < RY; ++r) {
+          float rsum = 0.f;
           float xl = shfl_left(q[L - 1][CC][r][V - 1]), xr = shfl_right(q[L - 1][CC][r][0]);
           if (first) xl = vxl;
           if (last) xr = vxr;
 #pragma unroll
           for (int j = 0; j < V; ++j) {
             BrickAcc<RY> acc{q[L - 1][CC], q[L - 1][ZM], q[L - 1][ZP], up, dn, xl, xr, r, j};
-            float res[1], unused = 0.f;
-            p.op(acc, res, unused);
+            float res[1], second = 0.f;
+            p.op(acc, res, second);
             o[r][j] = res[0];
+            if constexpr (MODE == kBrickAdjoint) rsum = fma_(second, ut[L - 1][r][j], rsum);
+          }
+          if constexpr (MODE == kBrickAdjoint) {
+            const float v = inside && (ok >> r & 1) ? rsum : 0.f;
+            const float n = add(sum, v), d = sub(n, sum);
+            low = add(low, add(sub(sum, sub(n, d)), sub(v, d)));
+            sum = n;
+          }
+        }
+        if constexpr (MODE == kBrickAdjoint) load_state(L, t + 1);
+        if constexpr (MODE == kBrickStates && L < K) {
+          if (unsigned(t - K - L) < unsigned(z1 - z0)) {
+            T* d = p.out[L - 1] + (zoff - L * plane + rowoff);
+#pragma unroll
+            for (int r = 0; r < RY; ++r)
+              if (ok >> r & 1) strip_store(d + int64_t(r) * nx, o[r]);
           }
         }
         if constexpr (L == K) {
@@ -286,6 +355,7 @@ struct Brick {
       if constexpr (K >= 3) level(StripTag<3>());
       if constexpr (K >= 4) level(StripTag<4>());
       dst += plane;
+      zoff += plane;
       rd = (rd + G::ROWB) & (D * G::ROWB - 1);
       __syncthreads();
     };
@@ -304,12 +374,25 @@ struct Brick {
     run_to(StripTag<0>(), z1 + K > zhi ? nsteps - 2 * K - 2 : nsteps);
     run_to(StripTag<1>(), nsteps);
     cp_async_wait<0>();
+    if constexpr (MODE == kBrickAdjoint) {
+      // the block's sum in a fixed order
+      __shared__ double ws[G::THREADS / 32];
+      double total = double(sum) + double(low);
+      for (int o = 16; o > 0; o >>= 1) total += __shfl_down_sync(0xffffffffu, total, o);
+      if (threadIdx.x % 32 == 0) ws[threadIdx.x / 32] = total;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        double s = 0.0;
+        for (int w = 0; w < G::THREADS / 32; ++w) s += ws[w];
+        p.partials[blockIdx.x] += s;
+      }
+    }
   }
 };
 
-template <class Op, class T, int K, int RY, int WY, int MINB, bool VEC>
-__global__ void __launch_bounds__(BrickGeom<T, K, RY, WY>::THREADS, MINB) brick3d_kernel(const __grid_constant__ BrickParams<Op, T> p) {
-  using B = Brick<Op, T, K, RY, WY, VEC>;
+template <class Op, class T, int K, int RY, int WY, int MODE, bool VEC>
+__global__ void __launch_bounds__(BrickGeom<T, K, RY, WY>::THREADS, 1) brick3d_kernel(const __grid_constant__ BrickParams<Op, T> p) {
+  using B = Brick<Op, T, K, RY, WY, MODE, VEC>;
   using G = typename B::G;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int ntiles = p.tiles_x * p.tiles_y;

@@ -30,10 +30,12 @@ template <int K> int brick_chunk(int nz, int tiles, int slots) {
   return bzc;
 }
 
-template <class Op, class T, int K> struct BrickRunner {
+template <class Op, class T, int K, int MODE = kBrickPlain> struct BrickRunner {
   using G = BrickGeom<T, K, kRY, kWY>;
-  template <bool VEC> static cudaError_t go(const StepArgs& a, const Op& op) {
-    auto kern = &brick3d_kernel<Op, T, K, kRY, kWY, 1, VEC>;
+  // outs: the output of every level (kBrickStates), else out[K-1] alone is used
+  template <bool VEC>
+  static cudaError_t go(const StepArgs& a, const Op& op, void* const* outs, const void* const* uts, int* blocks_out) {
+    auto kern = &brick3d_kernel<Op, T, K, kRY, kWY, MODE, VEC>;
     static bool ready = false;
     if (!ready) {
       const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(G::SMEM));
@@ -44,7 +46,11 @@ template <class Op, class T, int K> struct BrickRunner {
     std::memset(static_cast<void*>(&p), 0, sizeof(p));
     p.op = op;
     p.in = static_cast<const T*>(a.in[0]);
-    p.out = static_cast<T*>(a.out[0]);
+    for (int l = 0; l < K; ++l) {
+      p.out[l] = static_cast<T*>(outs ? outs[l] : a.out[0]);
+      if (uts) p.ut[l] = static_cast<const T*>(uts[l]);
+    }
+    p.partials = a.partials;
     p.g.nx = int(a.g.n[2]);
     p.g.ny = int(a.g.n[1]);
     p.g.nz = int(a.g.n[0]);
@@ -58,13 +64,15 @@ template <class Op, class T, int K> struct BrickRunner {
     const int tiles = p.tiles_x * p.tiles_y;
     p.zchunk = brick_chunk<K>(p.g.nz, tiles, strip_sms());
     const int blocks = tiles * ((p.g.nz + p.zchunk - 1) / p.zchunk);
+    if (blocks_out) *blocks_out = blocks;
+    if (MODE == kBrickAdjoint && (!a.partials || blocks > a.partial_count)) return cudaErrorInvalidValue;
     kern<<<blocks, G::THREADS, G::SMEM, a.stream>>>(p);
     count_launches(1);
     return cudaGetLastError();
   }
   static cudaError_t run(const StepArgs& a, const Op& op) {
-    if (strip_vec(a)) return go<true>(a, op);
-    if constexpr (sizeof(T) == 4) return go<false>(a, op);
+    if (strip_vec(a)) return go<true>(a, op, nullptr, nullptr, nullptr);
+    if constexpr (sizeof(T) == 4) return go<false>(a, op, nullptr, nullptr, nullptr);
     return cudaErrorNotSupported;
   }
 };
@@ -78,7 +86,32 @@ template <class Op> cudaError_t brick_op(const StepArgs& a, const Op& op) {
   return a.g.dtype == kF32 ? brick_t<Op, float>(a, op) : brick_t<Op, __nv_bfloat16>(a, op);
 }
 
+template <class T> cudaError_t states_t(const StepArgs& a, void* const* outs) {
+  const OpDiff7 op{a.s.prm[0]};
+  if (a.ksteps == 4) return BrickRunner<OpDiff7, T, 4, kBrickStates>::template go<true>(a, op, outs, nullptr, nullptr);
+  if (a.ksteps == 2) return BrickRunner<OpDiff7, T, 2, kBrickStates>::template go<true>(a, op, outs, nullptr, nullptr);
+  return cudaErrorNotSupported;
+}
+template <class T> cudaError_t adjoint_t(const StepArgs& a, const void* const* uts, int* blocks) {
+  const OpBrickAdjoint op{a.s.prm[0]};
+  if (a.ksteps == 2) return BrickRunner<OpBrickAdjoint, T, 2, kBrickAdjoint>::template go<true>(a, op, nullptr, uts, blocks);
+  return cudaErrorNotSupported;
+}
+
 }  // namespace
+
+cudaError_t launch_brick_states(const StepArgs& a, void* const* outs) {
+  return a.g.dtype == kF32 ? states_t<float>(a, outs) : states_t<__nv_bfloat16>(a, outs);
+}
+cudaError_t launch_brick_adjoint(const StepArgs& a, const void* const* uts, int* blocks) {
+  return a.g.dtype == kF32 ? adjoint_t<float>(a, uts, blocks) : adjoint_t<__nv_bfloat16>(a, uts, blocks);
+}
+bool brick_adjoint_supported(const StepArgs& a) {
+  StepArgs b = a;
+  b.adjoint = false;
+  b.ksteps = 2;
+  return a.s.kind == kDiff7 && strip_vec(a) && brick_supported(b);
+}
 
 bool brick_supported(const StepArgs& a) {
   const Geom& g = a.g;

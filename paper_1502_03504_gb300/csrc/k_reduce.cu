@@ -52,9 +52,12 @@ __global__ void __launch_bounds__(kThreads) loss_seed_kernel(const T* __restrict
   double acc = 0.0;
   for (int64_t i = blockIdx.x * int64_t(kThreads) + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * kThreads) {
-    const double d = double(to_c(u[i])) - double(to_c(tgt[i]));
+    const C_t<T> a = to_c(u[i]), b = to_c(tgt[i]);
+    const double d = double(a) - double(b);
     acc = __fma_rn(d, d, acc);
-    lam[i] = from_c<T>(C_t<T>(2.0 * d));
+    // 2 (a - b) in compute precision: one rounding, as of the FP64 difference,
+    // and two instructions fewer on the FP64 pipe that bounds this kernel
+    lam[i] = from_c<T>(mul(C_t<T>(2), sub(a, b)));
   }
   const double s = block_sum(acc, ws);
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
@@ -68,6 +71,12 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(const double* partia
   for (int i = threadIdx.x; i < count; i += kThreads) acc += partials[i];
   const double s = block_sum(acc, ws);
   if (threadIdx.x == 0) *result = accumulate ? *result + s : s;
+}
+
+// Zero FP64 values: a kernel rather than a memset, whose graph node would
+// belong to the allocation the graph was captured with.
+__global__ void __launch_bounds__(kThreads) zero_kernel(double* p, int count) {
+  for (int i = blockIdx.x * kThreads + threadIdx.x; i < count; i += gridDim.x * kThreads) p[i] = 0.0;
 }
 
 int blocks_for(int64_t n) {
@@ -106,6 +115,12 @@ cudaError_t launch_loss_seed(int dtype, const void* uT, const void* target, void
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_finalize(partials, b, loss, 0, s);
+}
+
+cudaError_t launch_zero(double* p, int count, cudaStream_t s) {
+  zero_kernel<<<(count + kThreads - 1) / kThreads, kThreads, 0, s>>>(p, count);
+  count_launches(1);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_finalize(const double* partials, int count, double* result, int accumulate,

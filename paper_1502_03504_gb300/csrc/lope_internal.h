@@ -123,6 +123,13 @@ cudaError_t launch_brick(const StepArgs& a);
 bool brick_supported(const StepArgs& a);
 int64_t brick_cells(const StepArgs& a);  // cells of the blocks that cover a plane, halo included
 constexpr int kBrickK = 4;
+// The adjoint's forms of the bricks (diff7, aligned rows): a.ksteps = 4 or 2
+// sweeps storing every state, the state after sweep l in outs[l-1]; and
+// a.ksteps = 2 steps of the transposed function backward in time, step l with
+// the state uts[l-1], its dL/dc sums added to a.partials.
+cudaError_t launch_brick_states(const StepArgs& a, void* const* outs);
+cudaError_t launch_brick_adjoint(const StepArgs& a, const void* const* uts, int* blocks);
+bool brick_adjoint_supported(const StepArgs& a);
 int strip_kmax_of(const StepArgs& a);
 constexpr int kStripUserK = 4;  // depth of run-time compiled functions
 // Run-time compiled local functions (jit.cu).
@@ -153,6 +160,7 @@ cudaError_t launch_reduce(int op, int dtype, const void* x, const void* y, int64
                           double* partials, double* result, cudaStream_t s);
 cudaError_t launch_loss_seed(int dtype, const void* uT, const void* target, void* lam, int64_t n,
                              double* partials, double* loss, cudaStream_t s);
+cudaError_t launch_zero(double* p, int count, cudaStream_t s);
 cudaError_t launch_finalize(const double* partials, int count, double* result, int accumulate,
                             cudaStream_t s);
 

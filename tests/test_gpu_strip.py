@@ -236,3 +236,44 @@ def test_bricks_write_only_their_output(lope):
         for b in bufs:
             assert bool((b[:guard] == sentinel).all()) and bool((b[guard + n:] == sentinel).all())
         assert torch.equal(u, keep)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("bc", [0, 1])
+@pytest.mark.parametrize("T,ckpt", [(23, 10), (13, 7), (6, 6), (9, 1)])
+def test_brick_adjoint_equals_one_step_kernels(lope, orc, dtype, bc, T, ckpt):
+    """diff7 on a grid large enough for the bricks: dL/du0 bitwise that of the
+    same steps one at a time (the forward sweeps of a function equal to its own
+    transpose), dL/dc the sum of <lambda, L u_t> to FP32 rounding of its terms."""
+    shape, c = (65, 256, 256), 0.1
+    u, _ = to_device(LI.uniform_field(1870, shape), dtype)
+    gT, _ = to_device(LI.normal_field(1871, shape), dtype)
+    st = lope.Stencil.builtin("diff7", c)
+    g = lope.Grid(shape, dtype, halo=1).set_boundaries([bc] * 3)
+    grad, gc = lope.vjp(g, st, u, gT, T, ckpt)
+    torch.cuda.synchronize()
+    lope.sync_status()
+    ref = _run(lope, g, st, gT, T, lope.Launch(DIRECT, 0, 0, 0, -1))
+    assert torch.equal(grad, ref)
+    # the sum in FP64 from the stored states: L u_t = (u_{t+1} - u_t) / c up to
+    # the rounding of the stored state, so evaluate L itself
+    def lap(x):
+        x = x.double()
+        if bc:
+            p = torch.nn.functional.pad(x, (1, 1, 1, 1, 1, 1))
+        else:
+            p = torch.nn.functional.pad(x[None, None], (1, 1, 1, 1, 1, 1), mode="circular")[0, 0]
+        s = p[2:, 1:-1, 1:-1] + p[:-2, 1:-1, 1:-1] + p[1:-1, 2:, 1:-1] + p[1:-1, :-2, 1:-1]
+        return s + p[1:-1, 1:-1, 2:] + p[1:-1, 1:-1, :-2] - 6.0 * x
+    lam, total, scale = gT, 0.0, 0.0
+    states = [u]
+    for _ in range(T - 1):
+        states.append(_run(lope, g, st, states[-1], 1, lope.Launch(DIRECT, 0, 0, 0, -1)))
+    for t in range(T - 1, -1, -1):
+        l = lap(lam)
+        total += float((l * states[t].double()).sum())
+        scale += float((lam.double().abs() * states[t].double().abs()).sum())
+        lam = _run(lope, g, st, lam, 1, lope.Launch(DIRECT, 0, 0, 0, -1))
+    # each term: 7 roundings of sums of at most 12 |lambda| |u|, then a chain of
+    # 4 FMAs and 2 adds in FP32 before FP64 takes over
+    assert abs(float(gc) - total) <= 12 * 13 * 2.0 ** -24 * scale
