@@ -49,7 +49,10 @@ inline int strip_sms() {
 }
 
 // Cut a grid into units for `slots` resident warps: as many chunks as fill
-// them once, but none shorter than the 2 K R rows it stages again.
+// them once, but none shorter than the 2 K R rows it stages again, unless the
+// grid is so small that some SMs would have no warp for each of their four
+// schedulers: then chunks of down to two rows (a launch's time is its longest
+// chunk's).
 inline StripCut strip_cut(const StripGrid& g, int valid, int kr, int slots) {
   StripCut c;
   c.strips = (g.nx + valid - 1) / valid;
@@ -58,7 +61,8 @@ inline StripCut strip_cut(const StripGrid& g, int valid, int kr, int slots) {
   const int ne = c.el + c.er, ni = c.strips - ne;
   const bool ylo = g.bc[0][0] == kDirichlet;
   constexpr int kNum = 2, kDen = 3;  // an edge chunk's share of an inner chunk's rows
-  const int most = g.ny / (2 * kr) > 1 ? g.ny / (2 * kr) : 1;
+  const int spread = std::min(g.ny / 2, 4 * strip_sms() / c.strips);
+  const int most = std::max(1, std::max(g.ny / (2 * kr), spread));
   // n chunks per inner strip, n * kDen / kNum per edge strip
   int n = int((int64_t(slots) * kNum) / (int64_t(ni) * kNum + int64_t(ne) * kDen));
   n = n < 1 ? 1 : n > most ? most : n;
