@@ -256,6 +256,45 @@ bool strip_choice(StepArgs a, Choice* c) {
   return true;
 }
 
+// FP64 grids of one field whose state stays in L2: the trapezoid tile and depth
+// with the least estimated time per sweep.  A launch lasts as long as its busiest
+// SM, which the FP64 pipe binds: in us, 2.38 + 0.64 per sweep + 0.0467 (5 terms;
+// 0.091 with 9) per window row of 32 points that the SM computes.  Fitted to 71
+// timings on GB300 (within 20 %; at each of the 14 grids the fastest tile and depth
+// of those timed is the one estimated so).  us for 40 sweeps, 64 x 16 at depth 4
+// (the choice of shorter calls) against the estimate's: jacobi5 256^2 162 -> 111
+// (64 x 8, depth 4: 128 blocks instead of 64 for 152 SMs), 100 x 300 164 -> 84 (32 x 8,
+// depth 4), 512^2 252 -> 224, star9r2 700 x 900 1190 -> 602 (32 x 8, depth 1).
+bool f64_choice(StepArgs a, Choice* c) {
+  const Geom& g = a.g;
+  if (g.ndim != 2 || g.nf != 1 || g.dtype != kF64 || a.s.stages != 1 || a.s.kind == kUser ||
+      npts(g) > (int64_t(1) << 20))
+    return false;
+  const int R = a.s.radius;
+  const int terms = a.s.kind == kLinear ? (2 * R + 1) * (2 * R + 1) : 4 * R + 1;
+  constexpr int64_t kSms = 152;
+  double best = 1e300;
+  for (int tx : {64, 32})
+    for (int ty : {16, 8})
+      for (int k : {4, 2, 1}) {
+        a.tile_x = tx;
+        a.tile_y = ty;
+        a.ksteps = k;
+        if (!trap2d_supported(a)) continue;
+        int64_t rows = 0;  // window rows of 32 points that a block computes
+        for (int s = 1; s <= k; ++s)
+          rows += int64_t((tx + 2 * R * (k - s) + 31) / 32) * (ty + 2 * R * (k - s));
+        const int64_t blocks = ((g.n[2] + tx - 1) / tx) * ((g.n[1] + ty - 1) / ty);
+        rows *= (blocks + kSms - 1) / kSms;
+        const double t = (2.38 + 0.64 * k + (0.0111 * terms - 0.0088) * double(rows)) / k;
+        if (t < best) {
+          best = t;
+          *c = {kPathTrap, tx, ty, k};
+        }
+      }
+  return best < 1e300;
+}
+
 Choice default_choice(const Geom& g, const StencilDesc& s, const void* const* in, int64_t nsteps,
                       int* err) {
   StepArgs a = base_args(g, s, err, nullptr);
@@ -270,17 +309,17 @@ Choice default_choice(const Geom& g, const StencilDesc& s, const void* const* in
   if (nsteps >= kStripSteps) {
     // Register strips and bricks, FP32 / BF16.  2D, measured on GB300 against the choices
     // below (which the same calls took before): jacobi5 FP32 7094^2 x20
-    // (unaligned rows) 1.65 -> 0.38 ms, 100 x 200 x20 51 -> 39 us; star9r2 FP32
+    // (unaligned rows) 1.65 -> 0.38 ms, 100 x 200 x20 51 -> 27 us; star9r2 FP32
     // 8192^2 x50 3.03 -> 1.72 ms; linear shallow water 4096^2 x3 x200 FP32 7.86
     // -> 2.60 ms, BF16 7.17 -> 2.45; RK3 nonlinear shallow water FP32 4096^2 x50
     // steps 14.2 -> 5.15 ms; a run-time compiled Gray-Scott FP32 4096^2 x100
-    // 3.99 -> 1.46 ms.  FP64 is bound by its arithmetic and stays below (256^2
-    // x100: 0.41 ms in trapezoid tiles, 0.46 in strips).
+    // 3.99 -> 1.46 ms.  FP64 is bound by its arithmetic and keeps to trapezoid
+    // tiles (256^2 x100: 0.28 ms, 0.46 in strips).
     StepArgs b = a;
     if (in)
       for (int f = 0; f < g.nf; ++f) b.in[f] = in[f];
     Choice c;
-    if (strip_choice(b, &c)) return c;
+    if (strip_choice(b, &c) || f64_choice(b, &c)) return c;
   }
   if (s.stages >= 2 && g.ndim == 2 && g.nf == 1 && g.dtype == kF32) {
     // Multi-stage steps of a single FP32 field: the fused trapezoid keeps the

@@ -140,6 +140,24 @@ def test_strips_default_plan_and_refusals(lope):
         lope.apply(lope.Grid(shape, "f64", halo=1), st, d, nsteps=4, launch=lope.Launch(STRIP, 0, 0, 4, -1))
 
 
+@pytest.mark.parametrize("shape", [(1, 1), (8, 32), (100, 300), (257, 255), (530, 515)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_double_default_plan_equals_direct(lope, shape):
+    """The FP64 tile and depth depend on the grid's size: the default plan's
+    result against one sweep per launch, also where the sweeps leave a rest."""
+    f = [to_device(LI.uniform_field(1840, shape, 0), "f64")[0]]
+    box = np.random.default_rng(5).uniform(-0.1, 0.1, (5, 5))
+    for st, halo in [(lope.Stencil.builtin("jacobi5", 0.2), 1), (lope.Stencil.builtin("star9r2", 0.1), 2),
+                     (lope.Stencil.linear(box), 2)]:
+        for bc, bv in BCS[:3]:
+            if bc[0] == 0 and min(shape) < halo:
+                continue
+            g = lope.Grid(shape, "f64", halo=halo).set_boundaries(bc, bv)
+            ref = _run(lope, g, st, f, 15, lope.Launch(DIRECT, 0, 0, 0, -1))
+            got = _run(lope, g, st, f, 15, None)
+            assert torch.equal(got[0], ref[0]), (shape, halo, bc)
+
+
 @pytest.mark.parametrize("shape", [(300, 200), (97, 203)], ids=lambda s: "x".join(map(str, s)))
 def test_strips_write_only_their_output(lope, shape):
     n = int(np.prod(shape))
