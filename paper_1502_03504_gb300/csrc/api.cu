@@ -1541,6 +1541,7 @@ lope_status lope_apply_batch(int n, const lope_grid* const* grids, const lope_st
   if (!plan) {
     plan = std::make_shared<BatchPlan>();
     int items = 0;
+    plan->dev.dirichlet = false;
     plan->host.resize(n);
     for (int i = 0; i < n; ++i) {
       const Geom& g = grids[i]->g;
@@ -1555,6 +1556,7 @@ lope_status lope_apply_batch(int n, const lope_grid* const* grids, const lope_st
         b.bval[0][sd] = g.bval[1][sd];
         b.bc[1][sd] = g.bc[2][sd];
         b.bval[1][sd] = g.bval[2][sd];
+        if (b.bc[0][sd] == kDirichlet || b.bc[1][sd] == kDirichlet) plan->dev.dirichlet = true;
       }
       b.tiles_x = mode ? 0 : (b.nx + tx - 1) / tx;
       b.first_item = items;

@@ -278,7 +278,7 @@ template <class T, int R, int NF, int K>
 std::string strip_name() {
   using Cfg = StripCfg<T, R, NF, K, 1>;
   char buf[256];
-  std::snprintf(buf, sizeof(buf), "&lope::strip2d_kernel<lope::UserOp, %s, %d, 1, %d, %d, %d, true>",
+  std::snprintf(buf, sizeof(buf), "&lope::strip2d_kernel<lope::UserOp, %s, %d, 1, %d, %d, %d, true, 0, true>",
                 std::is_same<T, float>::value ? "float" : "__nv_bfloat16", K, Cfg::D, Cfg::NWB,
                 Cfg::MINB);
   return buf;

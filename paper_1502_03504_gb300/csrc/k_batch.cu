@@ -128,8 +128,13 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(Op op, BatchPlanDe
 // whole vectors).  A persistent kernel whose warps claimed units from a counter
 // kept about 45 registers of its loop alive across the march and spilled it
 // (512 grids of sides 64..2048, jacobi5 x20, 5.9e8 points: 9.5 ms, with all
-// depths in one kernel 11.6 ms; this form 5.57 ms, the two-sweep shared-memory
-// tiles it replaced 12.5 ms).  Bound by instruction issue: 16 grids of 4096^2
+// depths in one kernel 11.6 ms; this form 5.09 ms, the two-sweep shared-memory
+// tiles it replaced 12.5 ms).  A batch with Dirichlet sides mixes masked and
+// plain units on an SM: at radius 1 all of them then run on packed pairs, whose
+// code is smaller (5.60 ms on scalars, 5.40 with pairs in the masked units only);
+// at radius 2 only the masked ones (256 odd grids x16: 3.93 ms, 4.05 on
+// scalars, 4.27 all packed).  A batch without Dirichlet sides runs a kernel
+// without masks, on scalars.  Bound by instruction issue: 16 grids of 4096^2
 // run 3.6e12 updates/s at depth 8; odd widths (element copies and stores)
 // and Dirichlet sides (masks) cost a quarter to a third.
 
@@ -150,12 +155,13 @@ __device__ __forceinline__ int find_grid_warp(const int* first, int n, int item)
 
 // One pass of depth K over the batch; pass 0 reads in, pass q > 0 what pass q-1
 // wrote.
-template <class Op, int K>
+template <class Op, int K, bool DIR>
 __global__ void __launch_bounds__(32 * kBatchWarps, 4)
     batch_strip_kernel(const __grid_constant__ Op op, const __grid_constant__ BatchPlanDev p,
                        int64_t pass) {
   using G = StripGeom<float, Op::R, K>;
   constexpr int D = strip_depth_index(K);
+  constexpr int PM = !DIR ? 0 : Op::R == 1 ? 2 : 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x / 32;
   const int u = blockIdx.x * kBatchWarps + warp;
@@ -181,9 +187,9 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 4)
   const int t = u - first[gi], c = t / strips, s = t - c * strips;
   const int y0 = c * p.chunk[D], y1 = min(g.ny, y0 + p.chunk[D]);
   if (g.nx % kStripV == 0)
-    Strip<Op, float, K, 1, kBatchRing, true>::run(op, in, out, g, s * G::VALID, y0, y1, ring, nullptr);
+    Strip<Op, float, K, 1, kBatchRing, true, PM>::template run<DIR>(op, in, out, g, s * G::VALID, y0, y1, ring, nullptr);
   else
-    Strip<Op, float, K, 1, kBatchRing, false>::run(op, in, out, g, s * G::VALID, y0, y1, ring, nullptr);
+    Strip<Op, float, K, 1, kBatchRing, false, PM>::template run<DIR>(op, in, out, g, s * G::VALID, y0, y1, ring, nullptr);
 }
 
 // Copy the plan's descriptors from page-locked host memory into the workspace
@@ -257,7 +263,8 @@ template <class Op, int K>
 cudaError_t launch_strip_pass(const Op& op, const BatchPlanDev& p, int64_t pass, cudaStream_t st) {
   constexpr size_t SMEM = size_t(kBatchWarps) * kBatchRing * StripGeom<float, Op::R, K>::ROWB;
   const int blocks = (p.units[strip_depth_index(K)] + kBatchWarps - 1) / kBatchWarps;
-  batch_strip_kernel<Op, K><<<blocks, 32 * kBatchWarps, SMEM, st>>>(op, p, pass);
+  if (p.dirichlet) batch_strip_kernel<Op, K, true><<<blocks, 32 * kBatchWarps, SMEM, st>>>(op, p, pass);
+  else batch_strip_kernel<Op, K, false><<<blocks, 32 * kBatchWarps, SMEM, st>>>(op, p, pass);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -200,6 +200,7 @@ struct BatchPlanDev {
   int units[kStripDepths];     // units of a pass
   int chunk[kStripDepths];     // rows per unit
   int64_t passes;
+  bool dirichlet;              // some grid has a Dirichlet side
 };
 // pinned: the grid list and (mode 1) the unit lists as they go into the
 // workspace from p.grids on, `bytes` long (a multiple of 16).

@@ -43,25 +43,55 @@ constexpr int kStripV = 4;  // columns per lane
 __device__ __forceinline__ float shfl_left(float v) { return __shfl_up_sync(0xffffffffu, v, 1); }
 __device__ __forceinline__ float shfl_right(float v) { return __shfl_down_sync(0xffffffffu, v, 1); }
 
-// Accessor of column p of a lane's row: q holds the 2R+1 rows of the level
-// below, row n in slot n mod (2R+1); C0 is the slot of the row being computed.
-// EAGER: the neighbouring lanes' columns of that row were fetched once (xl[i]:
-// column -1-i, xr[i]: column V+i); otherwise each tap that needs one shuffles
-// it.
-template <int NF, int NQ, int C0, bool EAGER>
+// A lane's V columns of a row.  Packed: two register pairs for the f32x2
+// instructions, pair j holding columns j and j + 2, so that a tap one column to
+// the side is the other pair for half of the columns and takes one move and a
+// shuffled value for the rest.
+template <bool PK> struct StripVal { using type = float; };
+template <> struct StripVal<true> { using type = F2; };
+template <bool PK> struct StripRow {
+  float w[kStripV];
+  __device__ __forceinline__ float get(int i) const { return w[i]; }
+  __device__ __forceinline__ void set(const float (&x)[kStripV]) {
+#pragma unroll
+    for (int i = 0; i < kStripV; ++i) w[i] = x[i];
+  }
+};
+template <> struct StripRow<true> {
+  F2 w[2];
+  __device__ __forceinline__ float get(int i) const { return i < 2 ? w[i].lo() : w[i - 2].hi(); }
+  __device__ __forceinline__ void set(const float (&x)[kStripV]) {
+    w[0] = F2::make(x[0], x[2]);
+    w[1] = F2::make(x[1], x[3]);
+  }
+};
+
+// Accessor of column p (packed: columns p and p + 2) of a lane's row: q holds
+// the 2R+1 rows of the level below, row n in slot n mod (2R+1); C0 is the slot of
+// the row being computed.  EAGER: the neighbouring lanes' columns of that row
+// were fetched once (xl[i]: column -1-i, xr[i]: column V+i); otherwise each tap
+// that needs one shuffles it.
+template <int NF, int NQ, int C0, bool EAGER, bool PK>
 struct StripAcc {
-  using C = float;
   static constexpr int V = kStripV;
-  const C (&q)[NQ][NF][V];
-  const C (&xl)[NF][NQ / 2];
-  const C (&xr)[NF][NQ / 2];
+  const StripRow<PK> (&q)[NQ][NF];
+  const float (&xl)[NF][NQ / 2];
+  const float (&xr)[NF][NQ / 2];
   int p;
-  __device__ __forceinline__ C operator()(int f, int dx, int dy, int) const {
-    const C(&w)[V] = q[(C0 + dy + NQ) % NQ][f];
+  __device__ __forceinline__ float at(const StripRow<PK>& w, int f, int i) const {
+    if (i < 0) return EAGER ? xl[f][-1 - i] : shfl_left(w.get(V + i));
+    if (i >= V) return EAGER ? xr[f][i - V] : shfl_right(w.get(i - V));
+    return w.get(i);
+  }
+  __device__ __forceinline__ auto operator()(int f, int dx, int dy, int) const {
+    const StripRow<PK>& w = q[(C0 + dy + NQ) % NQ][f];
     const int i = p + dx;
-    if (i < 0) return EAGER ? xl[f][-1 - i] : shfl_left(w[V + i]);
-    if (i >= V) return EAGER ? xr[f][i - V] : shfl_right(w[i - V]);
-    return w[i];
+    if constexpr (PK) {
+      if (i == 0 || i == 1) return w.w[i];
+      return F2::make(at(w, f, i), at(w, f, i + 2));
+    } else {
+      return at(w, f, i);
+    }
   }
   __device__ __forceinline__ int64_t gidx() const { return 0; }
 };
@@ -77,6 +107,14 @@ template <class T> __device__ __forceinline__ void strip_round(float (&w)[kStrip
       w[p + 1] = __uint_as_float(v & 0xffff0000u);
     }
   }
+}
+
+// A row's columns in order.
+__device__ __forceinline__ StripRow<false> strip_flat(const float (&o)[kStripV]) {
+  return {{o[0], o[1], o[2], o[3]}};
+}
+__device__ __forceinline__ StripRow<false> strip_flat(const F2 (&o)[2]) {
+  return {{o[0].lo(), o[1].lo(), o[0].hi(), o[1].hi()}};
 }
 
 // A lane's V values of a staged row (16 or 8 bytes of shared memory).
@@ -150,7 +188,9 @@ template <class T, int R, int K> struct StripGeom {
 // STG >= 2: the K = STG levels are the stages of one Runge-Kutta step: level l
 // >= 2 is a_l u + b_l E(level l-1), u read again from the ring, which keeps
 // STG R rows behind the newest for it.
-template <class Op, class T, int K, int STG, int D, bool VEC>
+// PM: which marches compute on packed pairs of columns, 0 none, 1 those with
+// masks, 2 all.
+template <class Op, class T, int K, int STG, int D, bool VEC, int PM>
 struct Strip {
   using C = float;
   using G = StripGeom<T, Op::R, K>;
@@ -164,12 +204,18 @@ struct Strip {
   // once per row.  The builtins of several fields read a few of theirs only.  A
   // run-time compiled function never shuffles inside its own body, whose
   // control flow is the user's.
-  static constexpr bool EAGER = Op::STAR && (NF == 1 || strip_user<Op>(0));
+  static constexpr bool USER = strip_user<Op>(0);
+  static constexpr bool EAGER = Op::STAR && (NF == 1 || USER);
 
   template <bool MASK>
   static __device__ __forceinline__ void march(const Op& op, const T* const* in, T* const* out,
                                                const StripGrid& g, int x0, int y0, int y1,
                                                unsigned char* ring, const Coef* rk) {
+    // Run-time compiled functions stay on scalars: their bodies may need them, and
+    // a packed product that feeds a sum may be contracted.
+    constexpr bool PK = !USER && (PM == 2 || (PM == 1 && MASK));
+    constexpr int NP = PK ? 2 : V;  // values of type W per row
+    using W = typename StripVal<PK>::type;
     const int lane = threadIdx.x & 31;
     const int nx = g.nx, ny = g.ny;
     const int x = x0 + (lane - G::HL) * V;  // this lane's first column
@@ -245,7 +291,7 @@ struct Strip {
       cp_async_commit();
     }
 
-    C q[K][NQ][NF][V];
+    StripRow<PK> q[K][NQ][NF];
     const int nv = lane < G::HL || lane >= 32 - G::HL ? 0 : max(0, min(V, nx - x));
     int64_t orow = int64_t(y0 - 2 * K * R) * nx + x;  // output offset of step t's stored row
     T* dst = out[0] + orow;
@@ -255,34 +301,38 @@ struct Strip {
       cp_async_wait<PF - 1>();
       if constexpr (!VEC) __syncwarp();
 #pragma unroll
-      for (int f = 0; f < NF; ++f)
-        strip_load(reinterpret_cast<const T*>(ring + f * RING + rd) + lane * V, q[0][PH][f]);
+      for (int f = 0; f < NF; ++f) {
+        C w[V];
+        strip_load(reinterpret_cast<const T*>(ring + f * RING + rd) + lane * V, w);
+        if constexpr (MASK && PK) mask(w, yb + t);
+        q[0][PH][f].set(w);
+      }
       if constexpr (!VEC) __syncwarp();
       if (t + PF < nsteps) copy_row((rd + PF * ROWB) & (RING - 1));
       cp_async_commit();
-      if constexpr (MASK) {
+      if constexpr (MASK && !PK) {
 #pragma unroll
-        for (int f = 0; f < NF; ++f) mask(q[0][PH][f], yb + t);
+        for (int f = 0; f < NF; ++f) mask(q[0][PH][f].w, yb + t);
       }
       auto level = [&](auto l_tag) {
         constexpr int L = decltype(l_tag)::value;
         constexpr int C0 = ((PH - L * R) % NQ + NQ) % NQ;
-        C o[NF][V];
+        W o[NF][NP];
         C xl[NF][R], xr[NF][R];
         if constexpr (EAGER) {
 #pragma unroll
           for (int f = 0; f < NF; ++f)
 #pragma unroll
             for (int i = 0; i < R; ++i) {
-              xl[f][i] = shfl_left(q[L - 1][C0][f][V - 1 - i]);
-              xr[f][i] = shfl_right(q[L - 1][C0][f][i]);
+              xl[f][i] = shfl_left(q[L - 1][C0][f].get(V - 1 - i));
+              xr[f][i] = shfl_right(q[L - 1][C0][f].get(i));
             }
         }
 #pragma unroll
-        for (int p = 0; p < V; ++p) {
-          StripAcc<NF, NQ, C0, EAGER> acc{q[L - 1], xl, xr, p};
-          C r[NF];
-          C unused = C(0);
+        for (int p = 0; p < NP; ++p) {
+          StripAcc<NF, NQ, C0, EAGER, PK> acc{q[L - 1], xl, xr, p};
+          W r[NF];
+          W unused = W(0.f);
           op(acc, r, unused);
 #pragma unroll
           for (int f = 0; f < NF; ++f) o[f][p] = r[f];
@@ -294,8 +344,10 @@ struct Strip {
             C b[V];
             strip_load(reinterpret_cast<const T*>(ring + f * RING + ((rd - L * R * ROWB) & (RING - 1))) + lane * V, b);
             if constexpr (MASK) mask(b, yb + t - L * R);
+            StripRow<PK> u;
+            u.set(b);
 #pragma unroll
-            for (int p = 0; p < V; ++p) o[f][p] = fma_(cb.get(C()), o[f][p], mul(ca.get(C()), b[p]));
+            for (int p = 0; p < NP; ++p) o[f][p] = fma_(cb.get(W()), o[f][p], mul(ca.get(W()), u.w[p]));
           }
         }
         if constexpr (L == K) {
@@ -304,19 +356,24 @@ struct Strip {
             for (int f = 0; f < NF; ++f) {
               T* d = NF == 1 ? dst : out[f] + orow;
               if constexpr (VEC) {
-                if (nv > 0) strip_store(d, o[f]);
+                if (nv > 0) strip_store(d, strip_flat(o[f]).w);
               } else {
-                strip_store_n(d, o[f], nv);
+                strip_store_n(d, strip_flat(o[f]).w, nv);
               }
             }
           }
         } else {
 #pragma unroll
           for (int f = 0; f < NF; ++f) {
-            strip_round<T>(o[f]);
-            if constexpr (MASK) mask(o[f], yb + t - L * R);
+            if constexpr (MASK || sizeof(T) == 2) {
+              StripRow<false> w = strip_flat(o[f]);
+              strip_round<T>(w.w);
+              if constexpr (MASK) mask(w.w, yb + t - L * R);
+              q[L][C0][f].set(w.w);
+            } else {
 #pragma unroll
-            for (int p = 0; p < V; ++p) q[L][C0][f][p] = o[f][p];
+              for (int p = 0; p < NP; ++p) q[L][C0][f].w[p] = o[f][p];
+            }
           }
         }
       };
@@ -349,9 +406,12 @@ struct Strip {
     cp_async_wait<0>();
   }
 
+  // DIR: the grid may have a Dirichlet side.
+  template <bool DIR>
   static __device__ __forceinline__ void run(const Op& op, const T* const* in, T* const* out,
                                              const StripGrid& g, int x0, int y0, int y1,
                                              unsigned char* ring, const Coef* rk) {
+    if constexpr (!DIR) return march<false>(op, in, out, g, x0, y0, y1, ring, rk);
     const bool dx = (g.bc[1][0] == kDirichlet && x0 - G::HL * V < 0) ||
                     (g.bc[1][1] == kDirichlet && x0 + G::VALID + G::HL * V > g.nx);
     const bool dy = (g.bc[0][0] == kDirichlet && y0 - K * R < 0) ||
@@ -412,10 +472,10 @@ namespace {
 
 // NWB warps per block, one unit each; neighbouring units cover neighbouring
 // strips of the same rows.
-template <class Op, class T, int K, int STG, int D, int NWB, int MINB, bool VEC>
+template <class Op, class T, int K, int STG, int D, int NWB, int MINB, bool VEC, int PM, bool DIR>
 __global__ void __launch_bounds__(32 * NWB, MINB)
     strip2d_kernel(const __grid_constant__ StripParams<Op, T> p) {
-  using S = Strip<Op, T, K, STG, D, VEC>;
+  using S = Strip<Op, T, K, STG, D, VEC, PM>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x / 32;
   const int u = blockIdx.x * NWB + warp;
@@ -423,7 +483,7 @@ __global__ void __launch_bounds__(32 * NWB, MINB)
   int s, y0, y1;
   strip_unit(p.cut, p.g.ny, u, &s, &y0, &y1);
   if (y0 >= y1) return;
-  S::run(p.op, p.in, p.out, p.g, s * S::G::VALID, y0, y1, smem_raw + warp * S::BYTES, p.rk);
+  S::template run<DIR>(p.op, p.in, p.out, p.g, s * S::G::VALID, y0, y1, smem_raw + warp * S::BYTES, p.rk);
 }
 
 }  // namespace

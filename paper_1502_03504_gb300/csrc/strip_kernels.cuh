@@ -35,6 +35,20 @@ template <class T, int R, int NF, int K, int STG> struct StripCfg {
   static constexpr int D = STG >= 2 ? 16 : 8;
   static constexpr int MINB = NF == 1 ? 4 : 2;
   static constexpr size_t SMEM = size_t(NWB) * NF * D * StripGeom<T, R, K>::ROWB;
+  // Which marches compute on packed pairs (PM of Strip).  A pair takes half the
+  // issue slots and twice the FMA pipe's time, and costs moves for the taps along
+  // x: BF16 gains everywhere, having moves for its conversions anyway (4096^2,
+  // 24 sweeps: linear shallow water 319 -> 290 us, nonlinear 804 -> 777, with
+  // Dirichlet sides 1306 -> 998), FP32 only with masks (nonlinear shallow water
+  // with Dirichlet sides 1171 -> 1073 us, star9r2 298 -> 278; without masks
+  // star9r2 8192^2 x50 1.70 -> 1.97 ms).  Element copies at depth 8 would spill.
+  static constexpr int pm(bool vec, bool dirichlet) {
+    return sizeof(T) == 2 ? 2 : !dirichlet || (!vec && K == 8) ? 0 : 1;
+  }
+  // Whether the kernel holds the masked march.  Without it one field gains (fewer
+  // registers: jacobi5 4096^2 x24 143 -> 138 us, BF16 star9r2 300^2 50 -> 39);
+  // three fields lose 2 to 3 % and keep it.
+  static constexpr bool masks(bool dirichlet) { return dirichlet || NF > 1; }
 };
 
 inline int strip_sms() {
@@ -87,6 +101,13 @@ inline bool strip_vec(const StepArgs& a) {
   return true;
 }
 
+inline bool strip_dirichlet(const StepArgs& a) {
+  for (int ax = 1; ax < 3; ++ax)
+    for (int sd = 0; sd < 2; ++sd)
+      if (a.g.bc[ax][sd] == kDirichlet) return true;
+  return false;
+}
+
 inline void strip_grid(const StepArgs& a, StripGrid* g) {
   g->nx = int(a.g.n[2]);
   g->ny = int(a.g.n[1]);
@@ -103,16 +124,17 @@ struct StripRunner {
   using Cfg = StripCfg<T, Op::R, Op::NF, K, STG>;
   using G = StripGeom<T, Op::R, K>;
   static constexpr size_t SMEM = Cfg::SMEM;
-  template <bool VEC> static auto kernel() {
-    return &strip2d_kernel<Op, T, K, STG, Cfg::D, Cfg::NWB, Cfg::MINB, VEC>;
+  template <bool VEC, bool DIR> static auto kernel() {
+    return &strip2d_kernel<Op, T, K, STG, Cfg::D, Cfg::NWB, Cfg::MINB, VEC,
+                           Cfg::pm(VEC, DIR), Cfg::masks(DIR)>;
   }
-  template <bool VEC> static cudaError_t occupancy(int* occ) {
+  template <bool VEC, bool DIR> static cudaError_t occupancy(int* occ) {
     static int o = -1;
     if (o < 0) {
-      cudaError_t e = cudaFuncSetAttribute(kernel<VEC>(), cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM));
+      cudaError_t e = cudaFuncSetAttribute(kernel<VEC, DIR>(), cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM));
       if (e != cudaSuccess) return e;
       int n = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel<VEC>(), 32 * Cfg::NWB, SMEM);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel<VEC, DIR>(), 32 * Cfg::NWB, SMEM);
       if (e != cudaSuccess) return e;
       o = n > 0 ? n : 1;
     }
@@ -134,24 +156,25 @@ struct StripRunner {
     p->cut = strip_cut(p->g, G::VALID, K * Op::R, occ * strip_sms() * Cfg::NWB);
     p->units = strip_units(p->cut);
   }
-  template <bool VEC> static cudaError_t go(const StepArgs& a, const Op& op) {
+  template <bool VEC, bool DIR> static cudaError_t go(const StepArgs& a, const Op& op) {
     int occ = 1;
-    cudaError_t e = occupancy<VEC>(&occ);
+    cudaError_t e = occupancy<VEC, DIR>(&occ);
     if (e != cudaSuccess) return e;
     StripParams<Op, T> p;
     std::memset(static_cast<void*>(&p), 0, sizeof(p));
     p.op = op;
     params(a, occ, &p);
-    kernel<VEC>()<<<(p.units + Cfg::NWB - 1) / Cfg::NWB, 32 * Cfg::NWB, SMEM, a.stream>>>(p);
+    kernel<VEC, DIR>()<<<(p.units + Cfg::NWB - 1) / Cfg::NWB, 32 * Cfg::NWB, SMEM, a.stream>>>(p);
     count_launches(1);
     return cudaGetLastError();
   }
   static cudaError_t run_vec(const StepArgs& a, const Op& op) {
-    return strip_vec(a) ? go<true>(a, op) : cudaErrorNotSupported;
+    if (!strip_vec(a)) return cudaErrorNotSupported;
+    return strip_dirichlet(a) ? go<true, true>(a, op) : go<true, false>(a, op);
   }
   static cudaError_t run(const StepArgs& a, const Op& op) {
-    if (strip_vec(a)) return go<true>(a, op);
-    if constexpr (sizeof(T) == 4) return go<false>(a, op);
+    if (strip_vec(a)) return run_vec(a, op);
+    if constexpr (sizeof(T) == 4) return strip_dirichlet(a) ? go<false, true>(a, op) : go<false, false>(a, op);
     return cudaErrorNotSupported;
   }
 };
