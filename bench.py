@@ -210,12 +210,12 @@ def run_reference(args):
 
 
 # ---------------------------------------------------------------- GPU arm
-KERNEL_SOURCES = ("k_tma.cu", "tma_kernels.cuh", "tma_device.cuh", "device_common.cuh",
-                  "lope_internal.h")
+KERNEL_SOURCES = ("strip_device.cuh", "strip_kernels.cuh", "k_strip.cuh", "k_strip_diff.cu",
+                  "brick_device.cuh", "k_brick.cu", "device_common.cuh", "lope_internal.h")
 
 
 def kernel_source_hash():
-    """Hash of the sources the TMA kernels are compiled from."""
+    """Hash of the sources the kernels of the step are compiled from."""
     h = hashlib.sha256()
     for name in KERNEL_SOURCES:
         with open(os.path.join(ROOT, "paper_1502_03504_gb300", "csrc", name), "rb") as fh:
@@ -382,7 +382,7 @@ def main():
            "unpipelined_value": upd_step * e2e_steps * ws / (serial_ms / 1e3)}
     del d3, d2
 
-    # ---------------- roofline of the dominant kernel (3D TMA z-march)
+    # ---------------- roofline of the dominant kernel (the 3D grid's)
     # The plan of each grid (path, temporal depth k, launches) comes from the
     # library.  One launch reads each point once and writes it once (8 B per
     # FP32 point) while it advances k sweeps, so its algorithmic bytes are
@@ -398,8 +398,11 @@ def main():
     ach3 = alg3 / launch3_s / 1e9
     ach2 = alg2 / launch2_s / 1e9
     tr = traffic_record()
-    name3 = ("tma3d_tb2s_kernel<OpDiff7, float> (512^3, two sweeps per launch)" if k3 == 2 else
-             "tma3d_kernel<OpDiff7, float> (512^3, one sweep per launch)")
+    path_names = {1: "TMA tiles", 2: "trapezoid tiles", 3: "direct", 4: "copied-plane march",
+                  5: "register strips / bricks"}
+    name3 = ("brick3d_kernel<OpDiff7, float>" if plan3.path == 5 else
+             "tma3d_tb2s_kernel<OpDiff7, float>" if k3 == 2 else "tma3d_kernel<OpDiff7, float>")
+    name3 += f" (512^3, {k3} sweeps per launch)"
     roofline = {"bound": "hbm", "achieved": ach3, "peak": peak, "unit": "GB/s",
                 "frac": ach3 / peak,
                 "traffic": tr.get(f"diff7_512_k{k3}_bytes_per_launch") if tr else None,
@@ -456,8 +459,8 @@ def main():
             "config": {"workload": WORKLOAD, "updates_per_step": upd_step,
                        "parallelism": f"replicas{ws}" if ws > 1 else "single",
                        "l2": "inputs larger than L2 (512 MiB and 256 MiB per buffer); no flush",
-                       "launch": f"lope_apply auto plan: TMA z-march (3D, {k3} sweeps per launch), "
-                                 f"TMA tiles (2D, {k2} sweep per launch)"},
+                       "launch": f"lope_apply auto plan: {path_names[plan3.path]} (3D, {k3} sweeps per "
+                                 f"launch), {path_names[plan2.path]} (2D, {k2} sweeps per launch)"},
             "e2e": e2e, "gpu_launches": launches, "clocks": clk, "roofline": roofline,
             "kernels": kernels, "cpu_baseline": cpu, "forms": forms,
         }
@@ -652,7 +655,7 @@ def form_swe_flux(L, LI, torch, dev, peak):
         del f, o, w
     res["bf16_speedup_vs_f32"] = res["f32"]["ms"] / res["bf16"]["ms"]
     res["workload"] = ("nonlinear flux-form C-grid shallow water (eta,u,v) 4096^2 periodic x200, "
-                       "dt 0.02, g 1, f 0.5, H 1; TMA tiles with box halo")
+                       "dt 0.02, g 1, f 0.5, H 1")
     return res
 
 
