@@ -311,7 +311,7 @@ Choice default_choice(const Geom& g, const StencilDesc& s, const void* const* in
     // below (which the same calls took before): jacobi5 FP32 7094^2 x20
     // (unaligned rows) 1.65 -> 0.38 ms, 100 x 200 x20 51 -> 27 us; star9r2 FP32
     // 8192^2 x50 3.03 -> 1.72 ms; linear shallow water 4096^2 x3 x200 FP32 7.86
-    // -> 2.60 ms, BF16 7.17 -> 2.45; RK3 nonlinear shallow water FP32 4096^2 x50
+    // -> 2.60 ms, BF16 7.17 -> 2.40; RK3 nonlinear shallow water FP32 4096^2 x50
     // steps 14.2 -> 5.15 ms; a run-time compiled Gray-Scott FP32 4096^2 x100
     // 3.99 -> 1.46 ms.  FP64 is bound by its arithmetic and keeps to trapezoid
     // tiles (256^2 x100: 0.28 ms, 0.46 in strips).

@@ -22,7 +22,9 @@
 // moves, 17 of the 52 instructions per level and row.  jacobi5 FP32 8192^2, per
 // sweep: 31 us with conditional levels on pairs of columns (packed f32x2
 // arithmetic), 25 us branch-free on scalars at K = 4, 17.7 us at K = 8, against
-// 56.8 us on the two-sweep shared-memory tiles.
+// 56.8 us on the two-sweep shared-memory tiles.  Packed arithmetic halves its issue
+// slots but not its time on the FMA pipe (K = 8: 138.5M -> 121.1M warp instructions,
+// 148 -> 162 us), so only marches with many other instructions use it (StripCfg::pm).
 //
 // The rows arrive in a private ring of shared memory per warp through
 // asynchronous copies (cp.async), PF rows ahead.  A lane's source column is
