@@ -120,6 +120,13 @@ lope_status check_pair(const lope_grid* grid, const lope_stencil* st) {
   return LOPE_OK;
 }
 
+// Whether [a, a + na) and [b, b + nb) share a byte.
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const char* x = static_cast<const char*>(a);
+  const char* y = static_cast<const char*>(b);
+  return x < y + nb && y < x + na;
+}
+
 // States each work buffer holds: two for the RK3 stage sequence (u1, u2), one
 // otherwise.
 int work_states(const StencilDesc& s) { return s.stages == 3 ? 2 : 1; }
@@ -144,11 +151,6 @@ lope_status check_fields(const Geom& g, const void* const* in, void* const* out,
     if (!aligned16(in[f]) || !aligned16(out[f])) return fail(LOPE_ERR_INVALID, "field pointer not 16-byte aligned");
     if (need_work && (!work[f] || !aligned16(work[f]))) return fail(LOPE_ERR_INVALID, "bad work pointer");
     const size_t bytes = size_t(npts(g)) * esize(g.dtype);
-    auto overlap = [&](const void* a, size_t na, const void* b, size_t nb) {
-      const char* x = static_cast<const char*>(a);
-      const char* y = static_cast<const char*>(b);
-      return x < y + nb && y < x + na;
-    };
     const size_t wbytes = bytes * size_t(wstates);
     // the input as read: the grid and its external halo planes
     const void* in_read = static_cast<const char*>(in[f]) - pad_lo;
@@ -801,6 +803,10 @@ lope_status reverse_impl(const lope_grid* grid, const lope_stencil* st, const vo
   probe.adjoint = false;
   probe.g = g;
   const bool brick = diffusion && g.ndim == 3 && aligned16(u0) && brick_adjoint_supported(probe) && strip_choice(probe, &sc);
+  // A gradient written over lambda_T (lope_vjp in place): with two steps in all, a
+  // pass of two would write cells of lambda_T that other blocks still read.
+  const size_t bytes = size_t(npts(g)) * esize(g.dtype);
+  const bool single = nsteps == 2 && overlap(lamT, bytes, grad_u0, bytes);
   int turn = 0;  // lambda buffers used in turn
   int blocks_used = 0;
   const void* lam = lamT;
@@ -834,7 +840,7 @@ lope_status reverse_impl(const lope_grid* grid, const lope_stencil* st, const vo
     }
     auto state = [&](int64_t j) { return j == 0 ? ck : static_cast<const void*>(seg(j)); };
     for (int64_t j = len - 1; j >= 0;) {
-      const int k = brick && j >= 1 ? 2 : 1;
+      const int k = brick && !single && j >= 1 ? 2 : 1;
       m += k;
       void* dst = m == nsteps ? grad_u0 : static_cast<void*>(ws + L.off_lam + size_t(turn) * L.field);
       turn ^= 1;

@@ -295,3 +295,28 @@ def test_brick_adjoint_equals_one_step_kernels(lope, orc, dtype, bc, T, ckpt):
     # each term: 7 roundings of sums of at most 12 |lambda| |u|, then a chain of
     # 4 FMAs and 2 adds in FP32 before FP64 takes over
     assert abs(float(gc) - total) <= 12 * 13 * 2.0 ** -24 * scale
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("T,ckpt", [(2, 2), (2, 5), (3, 3), (4, 2)])
+def test_brick_adjoint_in_place(lope, dtype, T, ckpt):
+    """lope_vjp with the gradient written over the upstream gradient: the values
+    of separate buffers (two steps in all would be one pass that reads cells of
+    one block while another writes them)."""
+    shape = (65, 256, 256)
+    u, _ = to_device(LI.uniform_field(1872, shape), dtype)
+    gT, _ = to_device(LI.normal_field(1873, shape), dtype)
+    st = lope.Stencil.builtin("diff7", 0.1)
+    g = lope.Grid(shape, dtype, halo=1)
+    want, gc = lope.vjp(g, st, u, gT, T, ckpt)
+    ws = torch.empty(lope.workspace_size(g, st, T, ckpt), dtype=torch.uint8, device="cuda")
+    got, gc2 = gT.clone(), torch.zeros(1, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    lope.lope_vjp(g.handle, st.handle, u.data_ptr(), got.data_ptr(), T, ckpt, 0, got.data_ptr(),
+                  gc2.data_ptr(), ws.data_ptr(), ws.numel(), 0)
+    torch.cuda.synchronize()
+    lope.sync_status()
+    assert torch.equal(got, want)
+    # dL/dc: the same terms, whichever steps share a pass, to the FP32 rounding of
+    # each (independent errors: L^T lambda rounds 7 times on sums of 12 |lambda|)
+    assert abs(float(gc2) - float(gc)) <= 100 * 2.0 ** -24 * float((T * gT.double().square().sum()).sqrt())
