@@ -206,6 +206,12 @@ struct Strip {
   // once per row.  The builtins of several fields read a few of theirs only.  A
   // run-time compiled function never shuffles inside its own body, whose
   // control flow is the user's.
+  // The builtins are plain arithmetic: what they compute from rows that have not
+  // come yet is dropped.  A run-time compiled function may loop or index by the
+  // values it reads, so its queues start out as copies of the first row and its
+  // last steps repeat the last one: it sees states and boundary values only.
+  // (Steps that leave out the incomplete levels instead doubled the code: 7.3 s
+  // to compile Gray-Scott, 4.3 this way.)
   static constexpr bool USER = strip_user<Op>(0);
   static constexpr bool EAGER = Op::STAR && (NF == 1 || USER);
 
@@ -294,6 +300,20 @@ struct Strip {
     }
 
     StripRow<PK> q[K][NQ][NF];
+    if constexpr (USER) {
+      cp_async_wait<PF - 1>();
+      if constexpr (!VEC) __syncwarp();
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        C w[V];
+        strip_load(reinterpret_cast<const T*>(ring + f * RING) + lane * V, w);
+        if constexpr (MASK) mask(w, yb);
+#pragma unroll
+        for (int l = 0; l < K; ++l)
+#pragma unroll
+          for (int n = 0; n < NQ; ++n) q[l][n][f].set(w);
+      }
+    }
     const int nv = lane < G::HL || lane >= 32 - G::HL ? 0 : max(0, min(V, nx - x));
     int64_t orow = int64_t(y0 - 2 * K * R) * nx + x;  // output offset of step t's stored row
     T* dst = out[0] + orow;
@@ -389,7 +409,7 @@ struct Strip {
       if constexpr (K >= 8) level(StripTag<8>());
       if constexpr (NF == 1) dst += nx;
       else orow += nx;
-      rd = (rd + ROWB) & (RING - 1);
+      if (!USER || t + 1 < nsteps) rd = (rd + ROWB) & (RING - 1);
     };
     // The step count is rounded up to the queue's period: the rows of the
     // first 2 K R steps whose level is not complete yet, and those past y1,

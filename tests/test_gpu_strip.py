@@ -120,6 +120,59 @@ def test_strips_run_time_compiled(lope, dtype):
                 _check(lope, g, st, f, T, k)
 
 
+# A function of NF fields and radius R whose every tap is checked: a value
+# outside [0.9, 2.1] sets the device error flag.  Its result is a mean, so states
+# and boundary values in [1, 2] stay there.  (C is float or a pair of floats.)
+CHECKED = """
+bool good = true;
+auto seen = [&](C v) {
+  const float* w = reinterpret_cast<const float*>(&v);
+  for (int i = 0; i < int(sizeof(C) / 4); ++i) good &= w[i] >= 0.9f && w[i] <= 2.1f;
+  return v;
+};
+for (int f = 0; f < NF; ++f) {
+  C s = seen(U((f + 1) % NF, 0, 0));
+  for (int k = 1; k <= R; ++k) {
+    s = add(s, add(seen(U(f, -k, 0)), seen(U(f, k, 0))));
+    s = add(s, add(seen(U(f, 0, -k)), seen(U(f, 0, k))));
+  }
+  out[f] = mul(P[0], s);
+}
+if (!good) raise_error(err, 2);
+"""
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("nf,radius", [(1, 1), (2, 1), (3, 1), (1, 2), (2, 2), (3, 2)])
+def test_strips_show_a_function_only_states_and_boundary_values(lope, dtype, nf, radius):
+    """A run-time compiled function of every shape, whatever rows its pipeline
+    fills or drains: no tap is anything but a state or a boundary value, and the
+    result is the direct kernel's."""
+    st = lope.Stencil.source(CHECKED, ndim=2, radius=radius, nfields=nf, params=[1.0 / (4 * radius + 1)])
+    for shape in ((2, 4), (3, 124), (40, 116), (67, 360), (513, 128)):
+        f = [1.0 + t for t in _fields(shape, dtype, 1, 1880)] * nf
+        f = [t.clone() for t in f]
+        for bc in ([0, 0], [1, 1], [1, 0]):
+            g = lope.Grid(shape, dtype, halo=radius, nfields=nf).set_boundaries(bc, [1.5 if b else 0.0 for b in bc])
+            for T, k in ((4, 4), (2, 2), (1, 1), (7, 4)):
+                _check(lope, g, st, f if nf > 1 else f[0:1], T, k)
+
+
+def test_strips_computed_taps(lope):
+    """Offsets computed at run time: inside the halo as on the direct kernel;
+    beyond it clamped and reported."""
+    g = lope.Grid((64, 128), "f32", halo=1)
+    u = torch.rand(64, 128, device="cuda")
+    body = "C s = C(0);\nfor (int d = -1; d <= %d; ++d) s = add(s, add(U(0, d, 0), U(0, 0, d)));\nout[0] = s;"
+    inside = lope.Stencil.source(body % 1, ndim=2, radius=1)
+    _check(lope, g, inside, [u], 7, 4)
+    beyond = lope.Stencil.source(body % 2, ndim=2, radius=1)
+    lope.apply(g, beyond, u, nsteps=4, launch=lope.Launch(STRIP, 0, 0, 4, -1))
+    with pytest.raises(lope.LopeError, match="outside its declared halo"):
+        lope.sync_status()
+    _check(lope, g, inside, [u], 4, 4)
+
+
 def test_strips_default_plan_and_refusals(lope):
     """Twelve sweeps or more take the strips; what they cannot run is refused."""
     shape = (64, 132)
