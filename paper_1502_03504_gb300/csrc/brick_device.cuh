@@ -82,12 +82,14 @@ enum : int {
   kBrickAdjoint = 2  // K steps of the transposed diffusion backward in time, each with its
                      // sum of (L^T lambda) u_t over the grid (dL/dc)
 };
-// Both forms of the adjoint are near HBM's rate.  256^3 FP32, us per launch: four
-// states stored 75 (320 MB; four sweeps one at a time 98); two adjoint steps 61
-// (256 MB; one at a time 2 x 41).  The states u_t go to registers one step ahead
-// of their use: staged two planes deep in shared memory they took 67, three steps
-// per pass 104, and with the sums in FP64 (its pipe runs one warp instruction in
-// about 19 cycles) 77 and 114.
+// 256^3 FP32, us per launch: four states stored 75 (320 MB; four sweeps one at a
+// time 98); two adjoint steps 63 (256 MB; one at a time 2 x 41).  The states u_t go
+// to registers one step ahead of their use: staged two planes deep in shared
+// memory that cost 6 more, and three steps per pass 43.
+// dL/dc is summed in FP64, whose pipe runs one warp instruction in about 19 cycles:
+// a conversion and an addition for each row of four cells made the launch 90 us.
+// So a thread gathers the row sums of three planes in a pair of floats without
+// loss (two-sum) before FP64 takes them; rows too large for a pair go to FP64 alone.
 
 // One step of lambda' = lambda + c L^T lambda; the second result is L^T lambda
 // (the operations of OpAdjDiffusion in the same order).
@@ -253,7 +255,10 @@ struct Brick {
       cp_async_commit();
     }
 
-    float sum = 0.f, low = 0.f;  // kBrickAdjoint: this thread's sum, and the rounding errors of it
+    // kBrickAdjoint: this thread's sum; the row sums not yet in it, and the
+    // rounding errors of their sum
+    double red = 0.0;
+    float sum = 0.f, low = 0.f;
     float q[K][3][RY][V];
     auto put_row = [&](float* d, const float (&w)[V]) {
       *reinterpret_cast<float4*>(d) = make_float4(w[0], w[1], w[2], w[3]);
@@ -294,13 +299,12 @@ struct Brick {
         strip_load(urow + (L - 1) * EXL, up);
         strip_load(drow + (L - 1) * EXL, dn);
         float o[RY][V];
-        // kBrickAdjoint: a chain of FMAs over a row's cells, added to the
-        // thread's sum with the addition's rounding error kept (two-sum), so
-        // the accumulation rounds like FP64 and leaves the slow FP64 pipe alone
+        // kBrickAdjoint: a chain of FMAs over each row's cells
+        float rsum[MODE == kBrickAdjoint ? RY : 1];
         const bool inside = MODE == kBrickAdjoint && unsigned(t - K - L) < unsigned(z1 - z0);
 #pragma unroll
         for (int r = 0; r < RY; ++r) {
-          float rsum = 0.f;
+          float chain = 0.f;
           float xl = shfl_left(q[L - 1][CC][r][V - 1]), xr = shfl_right(q[L - 1][CC][r][0]);
           if (first) xl = vxl;
           if (last) xr = vxr;
@@ -310,13 +314,24 @@ struct Brick {
             float res[1], second = 0.f;
             p.op(acc, res, second);
             o[r][j] = res[0];
-            if constexpr (MODE == kBrickAdjoint) rsum = fma_(second, ut[L - 1][r][j], rsum);
+            if constexpr (MODE == kBrickAdjoint) chain = fma_(second, ut[L - 1][r][j], chain);
           }
-          if constexpr (MODE == kBrickAdjoint) {
-            const float v = inside && (ok >> r & 1) ? rsum : 0.f;
-            const float n = add(sum, v), d = sub(n, sum);
-            low = add(low, add(sub(sum, sub(n, d)), sub(v, d)));
-            sum = n;
+          if constexpr (MODE == kBrickAdjoint) rsum[r] = inside && (ok >> r & 1) ? chain : 0.f;
+        }
+        if constexpr (MODE == kBrickAdjoint) {
+          float most = 0.f;
+#pragma unroll
+          for (int r = 0; r < RY; ++r) most = fmaxf(most, fabsf(rsum[r]));
+          if (most < 1.2676506e30f) {  // 2^100: no sum of a period's rows overflows
+#pragma unroll
+            for (int r = 0; r < RY; ++r) {
+              const float n = add(sum, rsum[r]), d = sub(n, sum);
+              low = add(low, add(sub(sum, sub(n, d)), sub(rsum[r], d)));
+              sum = n;
+            }
+          } else {
+#pragma unroll
+            for (int r = 0; r < RY; ++r) red += double(rsum[r]);
           }
         }
         if constexpr (MODE == kBrickAdjoint) load_state(L, t + 1);
@@ -368,6 +383,10 @@ struct Brick {
         step(StripTag<0>(), z_tag, t);
         step(StripTag<1>(), z_tag, t + 1);
         step(StripTag<2>(), z_tag, t + 2);
+        if constexpr (MODE == kBrickAdjoint) {
+          red += double(sum) + double(low);
+          sum = low = 0.f;
+        }
       }
     };
     run_to(StripTag<1>(), z0 - K < zlo ? 2 * K : 0);
@@ -377,7 +396,7 @@ struct Brick {
     if constexpr (MODE == kBrickAdjoint) {
       // the block's sum in a fixed order
       __shared__ double ws[G::THREADS / 32];
-      double total = double(sum) + double(low);
+      double total = red;
       for (int o = 16; o > 0; o >>= 1) total += __shfl_down_sync(0xffffffffu, total, o);
       if (threadIdx.x % 32 == 0) ws[threadIdx.x / 32] = total;
       __syncthreads();

@@ -373,3 +373,80 @@ def test_brick_adjoint_in_place(lope, dtype, T, ckpt):
     # dL/dc: the same terms, whichever steps share a pass, to the FP32 rounding of
     # each (independent errors: L^T lambda rounds 7 times on sums of 12 |lambda|)
     assert abs(float(gc2) - float(gc)) <= 100 * 2.0 ** -24 * float((T * gT.double().square().sum()).sqrt())
+
+
+def _dlap(x, bcs):
+    """L x in FP64 (Dirichlet 0 or periodic per axis), and the sum of the magnitudes
+    of its terms."""
+    p = x.double()
+    for ax in range(3):
+        if bcs[ax]:
+            z = torch.zeros_like(p.narrow(ax, 0, 1))
+            p = torch.cat([z, p, z], ax)
+        else:
+            p = torch.cat([p.narrow(ax, p.shape[ax] - 1, 1), p, p.narrow(ax, 0, 1)], ax)
+    def star(q):
+        return (q[2:, 1:-1, 1:-1] + q[:-2, 1:-1, 1:-1] + q[1:-1, 2:, 1:-1] + q[1:-1, :-2, 1:-1]
+                + q[1:-1, 1:-1, 2:] + q[1:-1, 1:-1, :-2])
+    return star(p) - 6.0 * x.double(), star(p.abs()) + 6.0 * x.double().abs()
+
+
+def _dc(lope, g, st, u, lam, T, bcs):
+    """dL/dc in FP64 from the stored states of single steps, the root of the sum of
+    the squared magnitudes of its terms, and dL/du0."""
+    one = lope.Launch(DIRECT, 0, 0, 0, -1)
+    states, total, square = [u], 0.0, 0.0
+    for _ in range(T - 1):
+        states.append(_run(lope, g, st, states[-1], 1, one))
+    for t in range(T - 1, -1, -1):
+        l, size = _dlap(lam, bcs)
+        total += float((l * states[t].double()).sum())
+        square += float((size * states[t].double()).square().sum())
+        lam = _run(lope, g, st, lam, 1, one)
+    return total, square ** 0.5, lam
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("shape,bcs", [((37, 380, 300), [1, 0, 1]), ((37, 380, 300), [0, 1, 0]),
+                                       ((130, 189, 204), [0, 0, 1]), ((130, 189, 204), [1, 1, 0])],
+                         ids=str)
+@pytest.mark.parametrize("T,ckpt", [(13, 7), (4, 4)])
+def test_brick_adjoint_counts_every_cell_once(lope, dtype, shape, bcs, T, ckpt):
+    """dL/dc on extents that are no multiple of a block's, sides of both kinds:
+    each term rounds at most 12 times (7 in L^T lambda, a chain of 4 FMAs, one
+    sum), independently, so four deviations of the sum are 4 * 12 / sqrt(3) *
+    2^-24 of the root sum square; a single missing cell is a hundred times that."""
+    u, _ = to_device(LI.uniform_field(1890, shape), dtype)
+    gT, _ = to_device(LI.normal_field(1891, shape), dtype)
+    st = lope.Stencil.builtin("diff7", 0.1)
+    g = lope.Grid(shape, dtype, halo=1).set_boundaries(bcs)
+    grad, gc = lope.vjp(g, st, u, gT, T, ckpt)
+    torch.cuda.synchronize()
+    lope.sync_status()
+    total, size, lam = _dc(lope, g, st, u, gT, T, bcs)
+    assert torch.equal(grad, lam)
+    assert abs(float(gc) - total) <= 28 * 2.0 ** -24 * size
+
+
+def test_brick_adjoint_sum_has_the_range_of_fp64(lope):
+    """Terms whose sum passes FP32's largest value while those of a row do not: the
+    second difference of lambda along x is +1 or -1, and u has its sign."""
+    shape, bcs, T = (65, 256, 256), [0, 0, 0], 2
+    s = np.where((np.arange(256) < 64) | (np.arange(256) >= 192), 1.0, -1.0)
+    slope = np.cumsum(s)
+    lam = np.concatenate([[0.0], np.cumsum(slope - slope.mean())[:-1]])  # exact: halves below 2^13
+    assert np.array_equal(np.roll(lam, -1) + np.roll(lam, 1) - 2 * lam, s)
+    gT = torch.from_numpy(lam * 2.0 ** 57).float().cuda().expand(shape).contiguous()
+    u = torch.from_numpy(s * 2.0 ** 66).float().cuda().expand(shape).contiguous()
+    st = lope.Stencil.builtin("diff7", 0.1)
+    g = lope.Grid(shape, "f32", halo=1).set_boundaries(bcs)
+    _, pairs = lope.vjp(g, st, u, gT, T, 2)   # one pass of two steps
+    _, single = lope.vjp(g, st, u, gT, T, 1)  # one step per pass: the same L^T lambda
+    torch.cuda.synchronize()
+    lope.sync_status()
+    # Only the sums differ: either rounds a term at most 5 times before FP64 takes it.
+    one = lope.Launch(DIRECT, 0, 0, 0, -1)
+    u1, lam1 = _run(lope, g, st, u, 1, one), _run(lope, g, st, gT, 1, one)
+    terms = sum(float((_dlap(l, bcs)[0] * v.double()).abs().sum()) for l, v in ((gT, u1), (lam1, u)))
+    assert float(single) > 1e40
+    assert abs(float(pairs) - float(single)) <= 10 * 2.0 ** -24 * 1.01 * terms
