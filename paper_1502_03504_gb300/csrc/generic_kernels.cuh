@@ -179,17 +179,10 @@ cudaError_t run_march(const StepArgs& a, const Op& op) {
   } else if constexpr (sizeof(T) == sizeof(C_t<T>)) {
     constexpr int smem = march_async_smem<C_t<T>, Op::NF, Op::R>();
     auto kern = &march3d_async_kernel<Op, T>;
-    static int per_sm = 0;  // resident blocks per SM, measured once per instance
-    if (per_sm == 0) {
-      if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-      }
-      int n = 0;
-      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, 256, smem);
-      if (e != cudaSuccess) return e;
-      per_sm = std::max(1, n);
-    }
+    static PerDevice memo;
+    int per_sm = 1;
+    const cudaError_t e = blocks_per_sm(memo, kern, 256, smem, &per_sm);
+    if (e != cudaSuccess) return e;
     if (!march_chunks(a.g, kAsyncX, kAsyncY, Op::R, per_sm, &blocks, &zchunk))
       return cudaErrorInvalidConfiguration;
     kern<<<blocks, 256, smem, a.stream>>>(op, a.g, in[0], in[1], in[2], out[0], out[1], out[2],

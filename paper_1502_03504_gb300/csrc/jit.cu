@@ -553,7 +553,7 @@ cudaError_t run_tb2(JitProgram& jp, const StepArgs& a, int dtype) {
       using Sh = Tb2sShape<T>;
       cudaError_t e = get_kernel(jp, dtype, tb2_index(false), Sh::SMEM, Sh::THREADS, &f, &occ);
       if (e != cudaSuccess) return e;
-      zmarch_geometry(a.g, p, &blocks, Sh::TX, Sh::TY, occ * sm_count());
+      zmarch_geometry(a.g, p, &blocks, Sh::TX, Sh::TY, occ * device_sms());
       if ((e = Sh::prepare(a, p, maps)) != cudaSuccess) return e;
       void* args[] = {&maps, &p};
       return launch(f, blocks, Sh::THREADS, Sh::SMEM, a.stream, args);

@@ -367,7 +367,7 @@ int batch_max_blocks(const StencilDesc& s, int dtype, int tile_x, int tile_y, in
       return 0;
     // resident blocks (the units are cut for them; nothing waits on another)
     const cudaError_t e = with_strip_op(s, [](auto) { return cudaSuccess; });
-    return e == cudaSuccess ? 4 * strip_sms() : 0;
+    return e == cudaSuccess ? 4 * device_sms() : 0;
   }
   if (!(s.kind == kJacobi5 || (s.kind == kLinear && s.star && s.ndim == 2 && s.radius == 1)))
     return 0;

@@ -36,12 +36,10 @@ template <class Op, class T, int K, int MODE = kBrickPlain> struct BrickRunner {
   template <bool VEC>
   static cudaError_t go(const StepArgs& a, const Op& op, void* const* outs, const void* const* uts, int* blocks_out) {
     auto kern = &brick3d_kernel<Op, T, K, kRY, kWY, MODE, VEC>;
-    static bool ready = false;
-    if (!ready) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(G::SMEM));
-      if (e != cudaSuccess) return e;
-      ready = true;
-    }
+    static PerDevice memo;
+    int occ = 0;
+    const cudaError_t e = blocks_per_sm(memo, kern, G::THREADS, G::SMEM, &occ);
+    if (e != cudaSuccess) return e;
     BrickParams<Op, T> p;
     std::memset(static_cast<void*>(&p), 0, sizeof(p));
     p.op = op;
@@ -62,7 +60,7 @@ template <class Op, class T, int K, int MODE = kBrickPlain> struct BrickRunner {
     p.tiles_x = brick_count(p.g.nx, G::BX, G::HL * kStripV, p.g.bc[2][0] == kDirichlet, p.g.bc[2][1] == kDirichlet);
     p.tiles_y = brick_count(p.g.ny, G::BY, K, p.g.bc[1][0] == kDirichlet, p.g.bc[1][1] == kDirichlet);
     const int tiles = p.tiles_x * p.tiles_y;
-    p.zchunk = brick_chunk<K>(p.g.nz, tiles, strip_sms());
+    p.zchunk = brick_chunk<K>(p.g.nz, tiles, device_sms());
     const int blocks = tiles * ((p.g.nz + p.zchunk - 1) / p.zchunk);
     if (blocks_out) *blocks_out = blocks;
     if (MODE == kBrickAdjoint && (!a.partials || blocks > a.partial_count)) return cudaErrorInvalidValue;

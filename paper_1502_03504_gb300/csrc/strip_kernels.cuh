@@ -8,6 +8,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "per_device.h"
 #include "strip_device.cuh"
 
 namespace lope {
@@ -51,17 +52,6 @@ template <class T, int R, int NF, int K, int STG> struct StripCfg {
   static constexpr bool masks(bool dirichlet) { return dirichlet || NF > 1; }
 };
 
-inline int strip_sms() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 1;
-  }
-  return n;
-}
-
 // Cut a grid into units for `slots` resident warps: as many chunks as fill
 // them once, but none shorter than the 2 K R rows it stages again, unless the
 // grid is so small that some SMs would have no warp for each of their four
@@ -75,7 +65,7 @@ inline StripCut strip_cut(const StripGrid& g, int valid, int kr, int slots) {
   const int ne = c.el + c.er, ni = c.strips - ne;
   const bool ylo = g.bc[0][0] == kDirichlet;
   constexpr int kNum = 2, kDen = 3;  // an edge chunk's share of an inner chunk's rows
-  const int spread = std::min(g.ny / 2, 4 * strip_sms() / c.strips);
+  const int spread = std::min(g.ny / 2, 4 * device_sms() / c.strips);
   const int most = std::max(1, std::max(g.ny / (2 * kr), spread));
   // n chunks per inner strip, n * kDen / kNum per edge strip
   int n = int((int64_t(slots) * kNum) / (int64_t(ni) * kNum + int64_t(ne) * kDen));
@@ -129,17 +119,8 @@ struct StripRunner {
                            Cfg::pm(VEC, DIR), Cfg::masks(DIR)>;
   }
   template <bool VEC, bool DIR> static cudaError_t occupancy(int* occ) {
-    static int o = -1;
-    if (o < 0) {
-      cudaError_t e = cudaFuncSetAttribute(kernel<VEC, DIR>(), cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM));
-      if (e != cudaSuccess) return e;
-      int n = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel<VEC, DIR>(), 32 * Cfg::NWB, SMEM);
-      if (e != cudaSuccess) return e;
-      o = n > 0 ? n : 1;
-    }
-    *occ = o;
-    return cudaSuccess;
+    static PerDevice memo;
+    return blocks_per_sm(memo, kernel<VEC, DIR>(), 32 * Cfg::NWB, SMEM, occ);
   }
   static void params(const StepArgs& a, int occ, StripParams<Op, T>* p) {
     for (int f = 0; f < Op::NF; ++f) {
@@ -153,7 +134,7 @@ struct StripRunner {
       p->rk[2 * (s - 2) + 1] = cb;
     }
     strip_grid(a, &p->g);
-    p->cut = strip_cut(p->g, G::VALID, K * Op::R, occ * strip_sms() * Cfg::NWB);
+    p->cut = strip_cut(p->g, G::VALID, K * Op::R, occ * device_sms() * Cfg::NWB);
     p->units = strip_units(p->cut);
   }
   template <bool VEC, bool DIR> static cudaError_t go(const StepArgs& a, const Op& op) {

@@ -9,6 +9,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "per_device.h"
 #include "tma_device.cuh"
 
 namespace lope {
@@ -48,17 +49,6 @@ cudaError_t encode(CUtensorMap* m, const void* base, int rank, const int64_t* n 
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
-int sm_count() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 1;
-  }
-  return n;
 }
 
 constexpr int kZWaves = 3;
@@ -121,7 +111,7 @@ struct TmaShape {
   static void geometry(const StepArgs& a, P& p, int* blocks, Occ&& occ) {
     const Geom& g = a.g;
     const bool wrap = g.bc[2][0] == kPeriodic || g.bc[1][0] == kPeriodic;
-    const int slots = occ(wrap) * sm_count();
+    const int slots = occ(wrap) * device_sms();
     if (RANK == 3) {
       zmarch_geometry(g, p, blocks, TX, TY, slots);
       return;
@@ -268,7 +258,7 @@ int tb2_2d_geometry(const Geom& g, P& p, int occ) {
   p.tiles_y = (p.ny + Sh2::TY - 1) / Sh2::TY;
   p.nunits = p.tiles_x * p.tiles_y;
   p.zchunk = 1;
-  return std::min(p.nunits, occ * sm_count());
+  return std::min(p.nunits, occ * device_sms());
 }
 
 // Whether the two-sweep kernels run this launch: in 3D a radius-1 star
@@ -324,17 +314,10 @@ struct TmaRunner {
   }
 
   template <bool TALL, bool WRAP> static int occupancy_w() {
-    static int occ = -1;
-    if (occ < 0) {
-      cudaFuncSetAttribute(kernel_w<TALL, WRAP>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(Sh<TALL>::SMEM));
-      int o = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kernel_w<TALL, WRAP>(), Sh<TALL>::THREADS,
-                                                        Sh<TALL>::SMEM) != cudaSuccess)
-        o = 1;
-      occ = o > 0 ? o : 1;
-    }
-    return occ;
+    static PerDevice memo;
+    int occ = 1;
+    const cudaError_t e = blocks_per_sm(memo, kernel_w<TALL, WRAP>(), Sh<TALL>::THREADS, Sh<TALL>::SMEM, &occ);
+    return e == cudaSuccess ? occ : 1;
   }
   template <bool TALL> static int occupancy(bool wrap) {
     return wrap ? occupancy_w<TALL, true>() : occupancy_w<TALL, false>();
@@ -377,19 +360,13 @@ struct TmaRunner {
     if constexpr (RANK == 3 && Op::R == 1 && Op::NF == 1 && Op::STAR && PAIR && !Op::REDUCES) {
       using Sh2 = Tb2Shape<T, TY, S>;
       auto kern = &tma3d_tb2_kernel<Op, T, Sh2::TX, Sh2::TY, Sh2::RY, Sh2::S>;
-      static int occ = -1;
-      if (occ < 0) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh2::SMEM));
-        int o = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, Sh2::THREADS, Sh2::SMEM) !=
-            cudaSuccess)
-          o = 1;
-        occ = o > 0 ? o : 1;
-      }
+      static PerDevice memo;
+      int occ = 1;
+      if (blocks_per_sm(memo, kern, Sh2::THREADS, Sh2::SMEM, &occ) != cudaSuccess) occ = 1;
       TmaParams<Op, T> p;
       p.op = op;
       int blocks = 0;
-      zmarch_geometry(a.g, p, &blocks, Sh2::TX, Sh2::TY, occ * sm_count());
+      zmarch_geometry(a.g, p, &blocks, Sh2::TX, Sh2::TY, occ * device_sms());
       if (blocks_out) *blocks_out = blocks;
       TmaMaps<1> maps;
       cudaError_t e = Sh2::prepare(a, p, maps);
@@ -410,15 +387,9 @@ struct TmaRunner {
     if constexpr (RANK == 2 && Op::R <= 2 && PAIR && !Op::REDUCES) {
       using Sh2 = Tb2Shape2D<T, Op::R, RY, Op::NF>;
       auto kern = &tma2d_tb2_kernel<Op, T, Sh2::TY, Sh2::RY, Sh2::S, WRAP>;
-      static int occ = -1;
-      if (occ < 0) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh2::SMEM));
-        int o = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, Sh2::THREADS, Sh2::SMEM) !=
-            cudaSuccess)
-          o = 1;
-        occ = o > 0 ? o : 1;
-      }
+      static PerDevice memo;
+      int occ = 1;
+      if (blocks_per_sm(memo, kern, Sh2::THREADS, Sh2::SMEM, &occ) != cudaSuccess) occ = 1;
       TmaParams<Op, T> p;
       p.op = op;
       const int blocks = tb2_2d_geometry<Sh2>(a.g, p, occ);
@@ -445,17 +416,13 @@ struct TmaRunner {
       constexpr int TX = Sh::TX, TY = Sh::TY, THREADS = Sh::THREADS;
       constexpr size_t SMEM = Sh::SMEM;
       auto kern = &tma3d_tb2s_kernel<Op, T, TX, TY, Sh::RY, Sh::S>;
-      static int occ = -1;
-      if (occ < 0) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM));
-        int o = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, THREADS, SMEM) != cudaSuccess) o = 1;
-        occ = o > 0 ? o : 1;
-      }
+      static PerDevice memo;
+      int occ = 1;
+      if (blocks_per_sm(memo, kern, THREADS, SMEM, &occ) != cudaSuccess) occ = 1;
       TmaParams<Op, T> p;
       p.op = op;
       int blocks = 0;
-      zmarch_geometry(a.g, p, &blocks, TX, TY, occ * sm_count());
+      zmarch_geometry(a.g, p, &blocks, TX, TY, occ * device_sms());
       if (blocks_out) *blocks_out = blocks;
       TmaMaps<1> maps;
       cudaError_t e = Sh::prepare(a, p, maps);
@@ -531,17 +498,10 @@ struct CaRunner {
     return Sh<TALL>::THREADS - 32 + 32 * NPW;
   }
   template <bool TALL> static int occupancy() {
-    static int occ = -1;
-    if (occ < 0) {
-      cudaFuncSetAttribute(kernel<TALL>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(smem<TALL>()));
-      int o = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kernel<TALL>(), threads<TALL>(),
-                                                        smem<TALL>()) != cudaSuccess)
-        o = 1;
-      occ = o > 0 ? o : 1;
-    }
-    return occ;
+    static PerDevice memo;
+    int occ = 1;
+    const cudaError_t e = blocks_per_sm(memo, kernel<TALL>(), threads<TALL>(), smem<TALL>(), &occ);
+    return e == cudaSuccess ? occ : 1;
   }
   template <bool TALL>
   static cudaError_t run_t(const StepArgs& a, const Op& op, int zchunk, int blocks) {
