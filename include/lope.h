@@ -255,9 +255,13 @@ lope_status lope_plan(const lope_grid* grid, const lope_stencil* stencil, const 
                       lope_launch* plan, int64_t* launches);
 
 /* Time candidate launch choices on the caller's buffers (out and work are
- * overwritten) and remember the fastest for this grid shape, dtype, stencil and
- * boundary; later lope_apply calls use it.  *best receives the choice and
- * *best_ms its time for nsteps.  Synchronises the stream. */
+ * overwritten): one sweep per launch on the tiles, marches and direct kernel,
+ * trapezoid tiles of several shapes and depths, and path 5 in 3D and in 2D from
+ * 2^20 points on.  *best receives the fastest and *best_ms its time for nsteps.
+ * Where it is faster than the plan that lope_apply makes by itself for nsteps, it
+ * is remembered for this grid shape, dtype, stencil and boundary and later
+ * lope_apply calls use it; else those keep making their own plan (and an earlier
+ * remembered choice is dropped).  Synchronises the stream. */
 lope_status lope_autotune(const lope_grid* grid, const lope_stencil* stencil,
                           const void* const* in, void* const* out, void* const* work,
                           int64_t nsteps, lope_launch* best, double* best_ms, void* cuda_stream);
@@ -305,12 +309,14 @@ lope_status lope_apply_batch(int n, const lope_grid* const* grids, const lope_st
                              size_t workspace_bytes, void* cuda_stream);
 
 /* Batch autotuner: times the batched launch over the register strips (where
- * they apply, from 2^20 points on) and the trapezoid tiles of shapes {128, 64} x {32, 16}
- * and temporal depths {1, 2, 4, 5} on the caller's buffers (out and work
- * are overwritten), stores the fastest for this batch (grid extents and
- * boundaries, dtype, stencil) and returns it in *best (*best_ms its time for
- * nsteps).  Later lope_apply_batch calls with cfg NULL (or zero tile/depth) on
- * a batch with the same signature use it.  Synchronises the stream. */
+ * they apply, for radius 1 from 2^20 points on) and the trapezoid tiles of shapes
+ * {128, 64} x {32, 16} and temporal depths {1, 2, 4, 5} on the caller's buffers
+ * (out and work are overwritten) and returns the fastest in *best (*best_ms its
+ * time for nsteps).  Where it is faster than the batch's own plan, it is stored
+ * for this batch (grid extents and boundaries, dtype, stencil), and later
+ * lope_apply_batch calls with cfg NULL (or zero tile/depth) on a batch with the
+ * same signature use it; else those keep the batch's plan.  Synchronises the
+ * stream. */
 lope_status lope_autotune_batch(int n, const lope_grid* const* grids, const lope_stencil* stencil,
                                 const void* const* in, void* const* out, void* const* work,
                                 int64_t nsteps, void* workspace, size_t workspace_bytes,

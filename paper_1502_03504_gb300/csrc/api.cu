@@ -297,8 +297,9 @@ bool f64_choice(StepArgs a, Choice* c) {
   return best < 1e300;
 }
 
+// tuned: a choice remembered by the autotuner comes first.
 Choice default_choice(const Geom& g, const StencilDesc& s, const void* const* in, int64_t nsteps,
-                      int* err) {
+                      int* err, bool tuned = true) {
   StepArgs a = base_args(g, s, err, nullptr);
   for (int f = 0; f < g.nf; ++f) a.in[f] = reinterpret_cast<const void*>(uintptr_t(256));
   {
@@ -306,7 +307,7 @@ Choice default_choice(const Geom& g, const StencilDesc& s, const void* const* in
     // used when it can run this grid
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(tune_key(g, s));
-    if (it != g_tune.end() && choice_supported(a, it->second)) return it->second;
+    if (tuned && it != g_tune.end() && choice_supported(a, it->second)) return it->second;
   }
   if (nsteps >= kStripSteps) {
     // Register strips and bricks, FP32 / BF16.  2D, measured on GB300 against the choices
@@ -946,6 +947,18 @@ int batch_strip_units(const std::vector<BatchGrid>& grids, int radius, int k, in
   return int(u);
 }
 
+// The batch's plan where no choice is remembered: the register strips for FP32 star
+// functions of radius 1-2 (jacobi5, star9r2, linear star tables), else trapezoid
+// tiles of 64 x 32, four sweeps per pass.
+bool batch_strips(const StencilDesc& s, int dtype) {
+  return dtype == kF32 && s.star && s.radius <= 2 &&
+         (s.kind == kJacobi5 || s.kind == kStar9r2 || s.kind == kLinear);
+}
+Choice batch_choice(const lope_grid* const* grids, const StencilDesc& s) {
+  if (!batch_strips(s, grids[0]->g.dtype)) return {kPathTrap, 64, 32, 4};
+  return {kPathStrip, 0, 0, strip_kmax_of(base_args(grids[0]->g, s, nullptr, nullptr))};
+}
+
 // Batch autotuner cache: the fastest (tile, depth) per batch signature (grid
 // shapes and boundaries, dtype, stencil), filled by lope_autotune_batch.
 using BatchSig = std::vector<int64_t>;
@@ -1400,35 +1413,56 @@ lope_status lope_autotune(const lope_grid* grid, const lope_stencil* stencil,
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const Geom& g = grid->g;
   std::vector<lope_launch> cands;
+  const lope_launch strips = {kPathStrip, 0, 0,
+                              stencil->s.stages >= 2 ? 1 : strip_kmax_of(base_args(g, stencil->s, nullptr, nullptr)), -1};
   cands.push_back({kPathTma, 0, 0, 1, -1});
   if (g.ndim == 2) {
-    if (npts(g) >= (int64_t(1) << 20)) {  // strips: worth their pipeline fill from here on
-      StepArgs probe = base_args(g, stencil->s, nullptr, nullptr);
-      cands.push_back({kPathStrip, 0, 0, stencil->s.stages >= 2 ? 1 : strip_kmax_of(probe), -1});
-    }
+    if (npts(g) >= (int64_t(1) << 20)) cands.push_back(strips);
     const int tiles[][2] = {{64, 32}, {128, 16}, {64, 16}, {32, 32}, {128, 32}};
     for (auto& t : tiles)
       for (int k : {1, 2, 3, 4, 6, 8}) cands.push_back({kPathTrap, t[0], t[1], k, -1});
   }
-  if (g.ndim == 3) cands.push_back({kPathMarch, 0, 0, 1, -1});
+  if (g.ndim == 3) {
+    cands.push_back({kPathMarch, 0, 0, 1, -1});
+    cands.push_back(strips);
+  }
   cands.push_back({kPathDirect, 0, 0, 1, -1});
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
+  // ms of one call after another (the first is the support check), < 0 if it fails
+  auto time = [&](const lope_launch& c) {
+    if (apply_impl(grid, stencil, in, out, work, nsteps, &c, st) != LOPE_OK) return -1.f;
+    cudaEventRecord(e0, st);
+    const lope_status r = apply_impl(grid, stencil, in, out, work, nsteps, &c, st);
+    cudaEventRecord(e1, st);
+    float ms = -1.f;
+    if (cudaEventSynchronize(e1) != cudaSuccess || r != LOPE_OK) return -1.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    return ms;
+  };
   double bms = 1e300;
   lope_launch bl = {0, 0, 0, 0, 0};
   for (const auto& c : cands) {
-    if (apply_impl(grid, stencil, in, out, work, nsteps, &c, st) != LOPE_OK) continue;  // warm-up / support check
-    cudaEventRecord(e0, st);
-    rs = apply_impl(grid, stencil, in, out, work, nsteps, &c, st);
-    cudaEventRecord(e1, st);
-    if (cudaEventSynchronize(e1) != cudaSuccess || rs != LOPE_OK) continue;
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, e0, e1);
-    if (ms < bms) {
+    const float ms = time(c);
+    if (ms >= 0.f && ms < bms) {
       bms = ms;
       bl = c;
     }
+  }
+  // The planner's own plan for this call is not slower than what is remembered: three
+  // timings of either in turn.
+  const Choice own = default_choice(g, stencil->s, in, nsteps, nullptr, false);
+  const lope_launch plan = {own.path, own.tile_x, own.tile_y, own.k, -1};
+  bool faster = bl.path != 0;
+  if (faster) {
+    float cand = 1e30f, mine = 1e30f;
+    for (int r = 0; r < 3; ++r) {
+      const float x = time(bl), y = time(plan);
+      if (x >= 0.f) cand = std::min(cand, x);
+      if (y >= 0.f) mine = std::min(mine, y);
+    }
+    faster = cand < mine;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1436,7 +1470,10 @@ lope_status lope_autotune(const lope_grid* grid, const lope_stencil* stencil,
   if (bl.path == 0) return fail(LOPE_ERR_UNSUPPORTED, "no launch path supports this grid/stencil");
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune[tune_key(g, stencil->s)] = {bl.path, bl.tile_x, bl.tile_y, bl.tsteps > 0 ? bl.tsteps : 1};
+    if (faster)
+      g_tune[tune_key(g, stencil->s)] = {bl.path, bl.tile_x, bl.tile_y, bl.tsteps > 0 ? bl.tsteps : 1};
+    else
+      g_tune.erase(tune_key(g, stencil->s));
   }
   if (best) *best = bl;
   if (best_ms) *best_ms = bms;
@@ -1482,16 +1519,12 @@ lope_status lope_apply_batch(int n, const lope_grid* const* grids, const lope_st
     void* work1[1] = {work ? work[i] : nullptr};
     if ((rs = check_fields(grids[i]->g, in1, out1, work1, true)) != LOPE_OK) return rs;
   }
-  // The register strips (path 5; path 1 runs them two sweeps per pass) serve FP32
-  // star functions of radius 1-2 (jacobi5, star9r2, linear star tables) and are
-  // the default there; other batches take the trapezoid tiles (path 2, 64 x 32,
-  // four sweeps per pass).  A choice remembered by the batch autotuner comes
-  // first; cfg overrides either.
-  const bool strip_ok = dtype == kF32 && s.star && s.radius <= 2 &&
-                        (s.kind == kJacobi5 || s.kind == kStar9r2 || s.kind == kLinear);
+  // The plan of the batch, a choice remembered by the batch autotuner before it; cfg
+  // overrides either (path 1 runs the strips two sweeps per pass).
+  const bool strip_ok = batch_strips(s, dtype);
   StepArgs probe = base_args(grids[0]->g, s, nullptr, nullptr);
   const int kmax = strip_kmax_of(probe);
-  Choice tuned = strip_ok ? Choice{kPathStrip, 0, 0, kmax} : Choice{kPathTrap, 64, 32, 4};
+  Choice tuned = batch_choice(grids, s);
   if (!cfg || cfg->path == kPathAuto || cfg->tile_x <= 0 || cfg->tile_y <= 0 || cfg->tsteps <= 0) {
     std::lock_guard<std::mutex> lk(g_btune_mu);
     auto it = g_btune.find(batch_sig(n, grids, s));
@@ -1647,44 +1680,58 @@ lope_status lope_autotune_batch(int n, const lope_grid* const* grids, const lope
   double bms = 1e300;
   lope_launch bl = {0, 0, 0, 0, 0};
   lope_status last = LOPE_OK;
+  // ms of one call after another (the first builds the plan's graph), < 0 if it fails
+  auto time = [&](const lope_launch& c) {
+    auto run = [&] {
+      return last = lope_apply_batch(n, grids, stencil, in, out, work, nsteps, &c, workspace,
+                                     workspace_bytes, cuda_stream);
+    };
+    if (run() != LOPE_OK) return -1.f;
+    cudaEventRecord(e0, st);
+    run();
+    cudaEventRecord(e1, st);
+    float ms = -1.f;
+    if (cudaEventSynchronize(e1) != cudaSuccess || last != LOPE_OK) return -1.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    return ms;
+  };
   std::vector<lope_launch> cands;
-  {
-    // Strips from 2^20 points on; batches below fit in a few trapezoid tiles
-    // per block.
-    int64_t pts = 0;
-    for (int i = 0; i < n; ++i)
-      if (grids[i]) pts += npts(grids[i]->g);
-    if (pts >= (int64_t(1) << 20) && grids[0]) {
-      StepArgs probe = base_args(grids[0]->g, stencil->s, nullptr, nullptr);
-      cands.push_back({kPathStrip, 0, 0, strip_kmax_of(probe), -1});
-    }
-  }
+  int64_t pts = 0;
+  for (int i = 0; i < n; ++i)
+    if (grids[i]) pts += npts(grids[i]->g);
+  // the only form of a radius-2 function
+  if (grids[0] && (pts >= (int64_t(1) << 20) || stencil->s.radius > 1))
+    cands.push_back({kPathStrip, 0, 0, strip_kmax_of(base_args(grids[0]->g, stencil->s, nullptr, nullptr)), -1});
   for (const auto& t : tiles)
     for (int k : {1, 2, 4, 5}) cands.push_back({kPathTrap, t[0], t[1], k, -1});
   for (const auto& c : cands) {
-    // first call builds and caches the plan's graph; the second is timed
-    if ((last = lope_apply_batch(n, grids, stencil, in, out, work, nsteps, &c, workspace,
-                                 workspace_bytes, cuda_stream)) != LOPE_OK)
-      continue;
-    cudaEventRecord(e0, st);
-    last = lope_apply_batch(n, grids, stencil, in, out, work, nsteps, &c, workspace,
-                            workspace_bytes, cuda_stream);
-    cudaEventRecord(e1, st);
-    if (cudaEventSynchronize(e1) != cudaSuccess || last != LOPE_OK) continue;
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, e0, e1);
-    if (ms < bms) {
+    const float ms = time(c);
+    if (ms >= 0.f && ms < bms) {
       bms = ms;
       bl = c;
     }
   }
+  const lope_status status = last;
+  bool faster = bl.path != 0;  // than the batch's own plan: three timings of either in turn
+  if (faster) {
+    const Choice own = batch_choice(grids, stencil->s);
+    const lope_launch plan = {own.path, own.tile_x, own.tile_y, own.k, -1};
+    float cand = 1e30f, mine = 1e30f;
+    for (int r = 0; r < 3; ++r) {
+      const float x = time(bl), y = time(plan);
+      if (x >= 0.f) cand = std::min(cand, x);
+      if (y >= 0.f) mine = std::min(mine, y);
+    }
+    faster = cand < mine;
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (bl.path == 0) return last != LOPE_OK ? last : fail(LOPE_ERR_UNSUPPORTED, "no batched plan ran");
+  if (bl.path == 0) return status != LOPE_OK ? status : fail(LOPE_ERR_UNSUPPORTED, "no batched plan ran");
   g_last_error = "no error";
   {
     std::lock_guard<std::mutex> lk(g_btune_mu);
-    g_btune[batch_sig(n, grids, stencil->s)] = {bl.path, bl.tile_x, bl.tile_y, bl.tsteps};
+    if (faster) g_btune[batch_sig(n, grids, stencil->s)] = {bl.path, bl.tile_x, bl.tile_y, bl.tsteps};
+    else g_btune.erase(batch_sig(n, grids, stencil->s));
   }
   if (best) *best = bl;
   if (best_ms) *best_ms = bms;

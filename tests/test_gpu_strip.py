@@ -450,3 +450,43 @@ def test_brick_adjoint_sum_has_the_range_of_fp64(lope):
     terms = sum(float((_dlap(l, bcs)[0] * v.double()).abs().sum()) for l, v in ((gT, u1), (lam1, u)))
     assert float(single) > 1e40
     assert abs(float(pairs) - float(single)) <= 10 * 2.0 ** -24 * 1.01 * terms
+
+
+@pytest.mark.parametrize("shape,name,prm,T", [((100, 200), "jacobi5", [0.2], 20), ((64, 256, 256), "diff7", [0.1], 16),
+                                              ((130, 100, 130), "diff7", [0.1], 16)], ids=str)
+def test_autotuner_keeps_a_faster_plan_of_the_planner(lope, shape, name, prm, T):
+    """The strips and bricks run these calls in about half the time of the tiles:
+    after tuning they still do, with the same result."""
+    st = lope.Stencil.builtin(name, *prm)
+    g = lope.Grid(shape, "f32", halo=1).set_boundaries([1] * len(shape))
+    u = torch.rand(shape, device="cuda")
+    o, w = torch.empty_like(u), torch.empty_like(u)
+    want = _run(lope, g, st, u, T, None)
+    best, ms = lope.autotune(g, st, u, o, w, T)
+    assert ms > 0 and best.path in (1, 2, 3, 4, STRIP)
+    assert lope.plan(g, st, u, o, w, nsteps=T)[0].path == STRIP
+    assert torch.equal(_run(lope, g, st, u, T, None), want)
+
+
+@pytest.mark.parametrize("name,prm,halo", [("jacobi5", [0.2], 1), ("star9r2", [0.1], 2)])
+def test_batch_autotuner_keeps_a_faster_plan(lope, name, prm, halo):
+    """Likewise for a batch below 2^20 points (strips: one kernel per pass and one
+    for the descriptors; trapezoid tiles: two kernels).  Radius 2 has no other form."""
+    st = lope.Stencil.builtin(name, *prm)
+    shapes = [(64 + 15 * i, 300 - 13 * i) for i in range(16)]
+    grids = [lope.Grid(s, "f32", halo=halo) for s in shapes]
+    ins = [torch.rand(s, device="cuda") for s in shapes]
+    outs, works = [torch.empty_like(x) for x in ins], [torch.empty_like(x) for x in ins]
+
+    def kernels():
+        n = lope.launch_count()
+        lope.apply_batch(grids, st, ins, outs, works, nsteps=20)
+        return lope.launch_count() - n
+
+    before = kernels()
+    assert before > 2
+    best, ms = lope.autotune_batch(grids, st, ins, outs, works, 20)
+    assert ms > 0
+    assert kernels() == before
+    torch.cuda.synchronize()
+    lope.sync_status()
