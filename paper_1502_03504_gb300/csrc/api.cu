@@ -234,11 +234,65 @@ int64_t count_passes(const Choice& c, int64_t nsteps) {
 // query or log the plan of a short call see the path they always saw.
 constexpr int64_t kStripSteps = 12;
 
+// Depth of a 2D call in strips, or 0 where the plan of shorter calls is as fast.  The
+// strips gain nearly everywhere at their deepest; these shapes have so many
+// instructions per row, and masks at Dirichlet x sides on top, that tiles reading a
+// state from L2 hold against them.  In brackets: us for 12 sweeps, plan of shorter
+// calls / strips at the depth not taken (and at the one taken).
+int strip_depth(const StepArgs& a) {
+  const Geom& g = a.g;
+  const StencilDesc& s = a.s;
+  const int64_t n = npts(g);
+  const bool box2 = !s.star && s.radius == 2, f32 = g.dtype == kF32, user = s.kind == kUser;
+  const bool side_x = g.bc[2][0] == kDirichlet || g.bc[2][1] == kDirichlet;
+  const bool side = side_x || g.bc[1][0] == kDirichlet || g.bc[1][1] == kDirichlet;
+  StepArgs one = a;
+  one.ksteps = 1;
+  const bool tma = tma_supported(one);
+  if (s.stages >= 2) {
+    // BF16 radius-2 tables (RK3 1000^2 Dirichlet 169 / 294, 4096^2 periodic 1475 / 1654;
+    // RK2 periodic 934 / 840) and the nonlinear shallow water with masks (RK3 BF16
+    // 848^2 Dirichlet 186 / 241, FP32 1000^2 243 / 255).
+    if (box2 && !f32) return side ? n < (1 << 17) : s.stages == 2 || n < (1 << 19);
+    return !(s.kind == kSweFlux && s.stages == 3 && side_x && tma && n >= (1 << 19) && n < (1 << 21));
+  }
+  // The state is past the trapezoid's 8 MB and short of the two-sweep tiles' 2^22 points:
+  // one sweep per launch on the tiles, from L2.
+  const bool large = size_t(n) * esize(g.dtype) * size_t(g.nf) > (size_t(8) << 20);
+  const bool from_l2 = tma && large && n < (int64_t(1) << 22);
+  if (box2) {
+    // Depth 4 spills and loses to depth 2 (FP32 periodic 1000^2 111 / 105 (74), 3600 x
+    // 3603 749 / 460 (320)); with masks depth 2 loses, too, on small grids (500^2 56 /
+    // 86 (74)) and to the tiles (3000^2 200 / 325 (247)), but not on large rows TMA
+    // cannot stage (2000 x 2003 266 / 281 (174)).
+    if (!side) return from_l2 ? 0 : 2;
+    return n < (tma ? 1 << 19 : 1 << 20) || (tma && large) ? 0 : 2;
+  }
+  // Nonlinear shallow water (FP32 1000^2 Dirichlet 66 / 86, periodic 86 / 62), radius 2
+  // (9-point star 2000^2 68 / 74), run-time compiled functions of radius 2 or three
+  // BF16 fields (two fields of radius 2, FP32 1400^2, 68 / 117).
+  if (from_l2 && side_x && (s.radius == 2 || s.kind == kSweFlux || (user && g.nf == 3 && !f32))) return 0;
+  if (user && s.radius == 2 && g.nf == 3) {
+    // 240 registers of queues at depth 4: it spills (FP32 1000^2 periodic 78 / 123,
+    // 4096^2 704 / 521 (482); BF16 4096^2 698 / 736 (432); with masks on small grids
+    // depth 2 loses, too: 300^2, y sides Dirichlet, 56 / - (74)).
+    if ((from_l2 && n < (1 << 20)) || (side && n < (1 << 18))) return 0;
+    return 2;
+  }
+  if (user && s.radius == 2 && g.nf == 2 && side) return 2;  // FP32 4096^2 495 / 392 (345)
+  if (s.kind == kSweFlux && !tma && side && n < (1 << 19)) return 2;  // 600 x 603 72 / 93 (74)
+  return strip_kmax_of(a);
+}
+
 // The strip choice for a grid: where the strips (2D) or bricks (3D) take it and
 // measured faster than the other paths.
 bool strip_choice(StepArgs a, Choice* c) {
   a.ksteps = a.s.stages >= 2 ? 1 : strip_kmax_of(a);
   if (!strip_supported(a)) return false;
+  if (a.g.ndim == 2) {
+    a.ksteps = strip_depth(a);
+    if (a.ksteps == 0) return false;
+  }
   if (a.g.ndim == 3) {
     // Rows TMA cannot stage always gain (diff7 FP32, us per sweep: 100 x 333 x 77
     // 26.4 -> 6.8, 130 x 500 x 510 75.8 -> 34.1, 511^3 278 -> 105).  On rows it can,
