@@ -294,8 +294,9 @@ lope_status lope_tune_cache_load(const char* path, const char* gpu_name, int* lo
  * cfg may be NULL: the choice of the batch autotuner for this batch (see
  * lope_autotune_batch), else, for FP32 star functions of radius 1-2 (jacobi5,
  * star9r2, linear star tables), the register strips (cfg->path 5: any row
- * pitch, up to 8 sweeps per pass for radius 1, 4 for radius 2, tsteps chooses
- * 8 / 4, 2 or 1; cfg->path 1 runs them two sweeps per pass), and the trapezoid
+ * pitch, up to 8 sweeps per pass for radius 1, 4 for radius 2 (2 in a batch with a
+ * Dirichlet side), tsteps chooses 8 (radius 1), 4, 2 or 1; cfg->path 1 runs them two
+ * sweeps per pass), and the trapezoid
  * tiles otherwise (cfg->path 2: 64 x 32 tiles, depth 4; tile_x, tile_y and
  * tsteps choose another shape and depth).  Errors as lope_apply;
  * LOPE_ERR_TIMEOUT is reported by lope_sync_status if a bounded barrier wait

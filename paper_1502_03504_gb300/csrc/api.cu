@@ -1008,9 +1008,19 @@ bool batch_strips(const StencilDesc& s, int dtype) {
   return dtype == kF32 && s.star && s.radius <= 2 &&
          (s.kind == kJacobi5 || s.kind == kStar9r2 || s.kind == kLinear);
 }
-Choice batch_choice(const lope_grid* const* grids, const StencilDesc& s) {
+// Radius 2 with Dirichlet sides: two sweeps per pass, as a deeper pass fills its masked
+// units too long (us, two-sweep tiles of before / depth 4 / depth 2: star9r2 x20, 64
+// grids of sides 64..512 226 / 276 / 192, 128 of 200..1000 1275 / 1419 / 1062, 256 of
+// 64..2048 6795 / 7170 / 5179; half of them periodic 6490 / 5611 / 4517; all periodic
+// 6926 / 3686 / 4651).
+Choice batch_choice(int n, const lope_grid* const* grids, const StencilDesc& s) {
   if (!batch_strips(s, grids[0]->g.dtype)) return {kPathTrap, 64, 32, 4};
-  return {kPathStrip, 0, 0, strip_kmax_of(base_args(grids[0]->g, s, nullptr, nullptr))};
+  int k = strip_kmax_of(base_args(grids[0]->g, s, nullptr, nullptr));
+  for (int i = 0; s.radius == 2 && i < n; ++i)
+    for (int ax = 1; ax < 3; ++ax)
+      for (int sd = 0; sd < 2; ++sd)
+        if (grids[i]->g.bc[ax][sd] == kDirichlet) k = 2;
+  return {kPathStrip, 0, 0, k};
 }
 
 // Batch autotuner cache: the fastest (tile, depth) per batch signature (grid
@@ -1578,7 +1588,7 @@ lope_status lope_apply_batch(int n, const lope_grid* const* grids, const lope_st
   const bool strip_ok = batch_strips(s, dtype);
   StepArgs probe = base_args(grids[0]->g, s, nullptr, nullptr);
   const int kmax = strip_kmax_of(probe);
-  Choice tuned = batch_choice(grids, s);
+  Choice tuned = batch_choice(n, grids, s);
   if (!cfg || cfg->path == kPathAuto || cfg->tile_x <= 0 || cfg->tile_y <= 0 || cfg->tsteps <= 0) {
     std::lock_guard<std::mutex> lk(g_btune_mu);
     auto it = g_btune.find(batch_sig(n, grids, s));
@@ -1768,7 +1778,7 @@ lope_status lope_autotune_batch(int n, const lope_grid* const* grids, const lope
   const lope_status status = last;
   bool faster = bl.path != 0;  // than the batch's own plan: three timings of either in turn
   if (faster) {
-    const Choice own = batch_choice(grids, stencil->s);
+    const Choice own = batch_choice(n, grids, stencil->s);
     const lope_launch plan = {own.path, own.tile_x, own.tile_y, own.k, -1};
     float cand = 1e30f, mine = 1e30f;
     for (int r = 0; r < 3; ++r) {

@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(Op op, BatchPlanDe
 // tiles it replaced 12.5 ms).  A batch with Dirichlet sides mixes masked and
 // plain units on an SM: at radius 1 all of them then run on packed pairs, whose
 // code is smaller (5.60 ms on scalars, 5.40 with pairs in the masked units only);
-// at radius 2 only the masked ones (256 odd grids x16: 3.93 ms, 4.05 on
+// at radius 2 only the masked ones (256 odd grids x16 at depth 4: 3.93 ms, 4.05 on
 // scalars, 4.27 all packed).  A batch without Dirichlet sides runs a kernel
 // without masks, on scalars.  Bound by instruction issue: 16 grids of 4096^2
 // run 3.6e12 updates/s at depth 8; odd widths (element copies and stores)

@@ -490,3 +490,18 @@ def test_batch_autotuner_keeps_a_faster_plan(lope, name, prm, halo):
     assert kernels() == before
     torch.cuda.synchronize()
     lope.sync_status()
+
+
+@pytest.mark.parametrize("kinds,passes", [([0, 0], 3), ([0, 1], 5), ([1, 1], 5)])
+def test_depth_of_radius_two_batches(lope, kinds, passes):
+    """Nine sweeps of star9r2: 4 + 4 + 1 on periodic grids, 2 + 2 + 2 + 2 + 1 where a grid
+    has Dirichlet sides, after one kernel for the descriptors; each grid as alone."""
+    st = lope.Stencil.builtin("star9r2", 0.1)
+    shapes = [(70, 133), (300, 224)]
+    grids = [lope.Grid(s, "f32", halo=2).set_boundaries([k, k]) for s, k in zip(shapes, kinds)]
+    ins = [torch.rand(s, device="cuda") for s in shapes]
+    n = lope.launch_count()
+    outs = lope.apply_batch(grids, st, ins, nsteps=9)
+    assert lope.launch_count() - n == passes + 1
+    for g, u, o in zip(grids, ins, outs):
+        assert torch.equal(_run(lope, g, st, u, 9, lope.Launch(DIRECT, 0, 0, 0, -1)), o)
