@@ -229,6 +229,8 @@ int64_t count_passes(const Choice& c, int64_t nsteps) {
   return n;
 }
 
+constexpr int kSms = 152;  // of a GB300: plans are made without a CUDA call
+
 // The register strips serve calls of at least kStripSteps sweeps (or steps).
 // Shorter calls keep the plans documented for them (see lope.h): callers that
 // query or log the plan of a short call see the path they always saw.
@@ -300,12 +302,17 @@ bool strip_choice(StepArgs a, Choice* c) {
     // ones (a chunk's fill is 8 planes: 16 x 256 x 256 4.0 / 5.3) and those whose
     // blocks would be mostly halo; from 2^22 points on the bricks do better (64 x
     // 128 x 512 7.5 -> 5.9, 256^3 periodic 26.0 -> 13.5, 512^3 110 -> 73.6, BF16
-    // 512^3 123 -> 70.6).
-    StepArgs one = a;
+    // 512^3 123 -> 70.6).  Where two sweeps per launch run, the bricks need more than
+    // two fifths of the SMs' time on output (us for 15 sweeps, Dirichlet: 16 x 512^2 88
+    // -> 107 at a share of 0.36, 24 x 512^2 135 -> 139 at 0.40, 40 x 512^2 189 -> 185 at
+    // 0.44, 16 x 300 x 1000 156 -> 111 at 0.47).
+    StepArgs one = a, two = a;
     one.ksteps = 1;
+    two.ksteps = 2;
     const Geom& g = a.g;
     if (tma_supported(one) && (npts(g) < (int64_t(1) << 22) || g.n[0] < 16 ||
-                               brick_cells(a) > 2 * g.n[1] * g.n[2]))
+                               brick_cells(a) > 2 * g.n[1] * g.n[2] ||
+                               (tma_supported(two) && brick_share(a, kSms) < 0.4)))
       return false;
   }
   *c = {kPathStrip, 0, 0, a.ksteps};
@@ -328,7 +335,6 @@ bool f64_choice(StepArgs a, Choice* c) {
     return false;
   const int R = a.s.radius;
   const int terms = a.s.kind == kLinear ? (2 * R + 1) * (2 * R + 1) : 4 * R + 1;
-  constexpr int64_t kSms = 152;
   double best = 1e300;
   for (int tx : {64, 32})
     for (int ty : {16, 8})

@@ -15,7 +15,7 @@ constexpr int kRY = 4, kWY = 16;  // rows per thread, half-warps per block
 // z chunks: among the counts that keep a chunk at least as long as its
 // pipeline's fill, the one that maximises the busy fraction of the last wave
 // times the share of planes that are not fill.
-template <int K> int brick_chunk(int nz, int tiles, int slots) {
+template <int K> int brick_chunk(int nz, int tiles, int slots, double* share = nullptr) {
   double best = -1.0;
   int bzc = nz;
   const int most = std::max(1, std::min(nz / (2 * K), 4 * slots / tiles + 1));
@@ -27,6 +27,7 @@ template <int K> int brick_chunk(int nz, int tiles, int slots) {
       bzc = zc;
     }
   }
+  if (share) *share = best;
   return bzc;
 }
 
@@ -129,6 +130,17 @@ int64_t brick_cells(const StepArgs& a) {
   const Geom& g = a.g;
   return int64_t(G::BX) * brick_count(int(g.n[2]), G::BX, G::HL * kStripV, g.bc[2][0] == kDirichlet, g.bc[2][1] == kDirichlet) *
          G::BY * brick_count(int(g.n[1]), G::BY, kBrickK, g.bc[1][0] == kDirichlet, g.bc[1][1] == kDirichlet);
+}
+
+double brick_share(const StepArgs& a, int slots) {
+  using G = BrickGeom<float, kBrickK, kRY, kWY>;
+  const Geom& g = a.g;
+  const int tx = brick_count(int(g.n[2]), G::BX, G::HL * kStripV, g.bc[2][0] == kDirichlet, g.bc[2][1] == kDirichlet);
+  const int ty = brick_count(int(g.n[1]), G::BY, kBrickK, g.bc[1][0] == kDirichlet, g.bc[1][1] == kDirichlet);
+  if (tx == 1 || ty == 1) return 1.0;
+  double share = 0.0;
+  brick_chunk<kBrickK>(int(g.n[0]), tx * ty, slots, &share);
+  return share;
 }
 
 cudaError_t launch_brick(const StepArgs& a) {

@@ -122,6 +122,9 @@ bool strip_supported(const StepArgs& a);
 cudaError_t launch_brick(const StepArgs& a);
 bool brick_supported(const StepArgs& a);
 int64_t brick_cells(const StepArgs& a);  // cells of the blocks that cover a plane, halo included
+// Share of `slots` SMs' time that the blocks spend on planes they store (1 for a
+// single row or column of blocks).
+double brick_share(const StepArgs& a, int slots);
 constexpr int kBrickK = 4;
 // The adjoint's forms of the bricks (diff7, aligned rows): a.ksteps = 4 or 2
 // sweeps storing every state, the state after sweep l in outs[l-1]; and

@@ -73,6 +73,22 @@ def test_depth_of_long_calls(lope, fn, dtype, shape, bc, want):
     assert _plan(lope, shape, dtype, fn, bc) == want
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("shape,bc,want", [
+    ((16, 512, 512), [D, D, D], (TMA, 2)),
+    ((24, 512, 512), [P, D, D], (TMA, 2)),
+    ((40, 512, 512), [D, D, D], (STRIP, 4)),
+    ((16, 512, 512), [P, P, P], (STRIP, 4)),
+    ((16, 304, 1000), [D, D, D], (STRIP, 4)),
+    ((16, 4096, 64), [D, D, D], (STRIP, 4)),
+    ((64, 64, 64), [D, D, D], (TMA, 1)),
+], ids=str)
+def test_bricks_on_thin_grids(lope, dtype, shape, bc, want):
+    """Thin grids whose blocks leave half of the SMs idle keep two sweeps per launch
+    where those run (x and y sides Dirichlet)."""
+    assert _plan(lope, shape, dtype, "diff7", bc) == want
+
+
 @pytest.mark.parametrize("fn,dtype,shape,bc,scheme,path", [
     ("box2", "bf16", (1000, 1000), [D, D], "rk2", TMA),
     ("box2", "bf16", (1000, 1000), [P, P], "rk2", STRIP),
