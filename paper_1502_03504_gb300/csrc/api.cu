@@ -838,6 +838,22 @@ StencilDesc reflected(const StencilDesc& s) {
   return r;
 }
 
+// Whether two adjoint steps per pass beat single steps on the TMA tiles, which need no
+// halo code where x and y sides are Dirichlet (us per call of 30 steps, checkpoint
+// 10, single steps / passes of two: FP32 Dirichlet 65 x 256^2 785 / 811, 130 x 188 x
+// 204 981 / 951, 128 x 200 x 300 1401 / 1230, 256^3 2487 / 2182; BF16 65 x 256^2 801 /
+// 924, 256^3 2278 / 2595, 40 x 600^2 2753 / 2317; y sides periodic 65 x 256^2 885 / 932,
+// 256^3 2763 / 2621; all periodic 950 / 821, 2941 / 2487).
+bool brick_adjoint_faster(const StepArgs& a, bool tma) {
+  const Geom& g = a.g;
+  auto side = [&](int ax) { return g.bc[ax][0] == kDirichlet || g.bc[ax][1] == kDirichlet; };
+  const bool small = npts(g) < (int64_t(3) << 21);
+  if (!tma || !side(2)) return true;
+  if (g.dtype == kF32) return !(side(1) && small);
+  // BF16: where the blocks cover more than one and a half times the grid
+  return 2 * brick_cells(a) <= 3 * g.n[1] * g.n[2] || !(side(1) || small);
+}
+
 // Reverse sweep: lambda from `lamT` back to grad_u0, recomputing states from
 // checkpoints; dL/dc accumulated into per-block partials, finalised into gc.
 lope_status reverse_impl(const lope_grid* grid, const lope_stencil* st, const void* u0,
@@ -863,7 +879,8 @@ lope_status reverse_impl(const lope_grid* grid, const lope_stencil* st, const vo
   probe.in[0] = u0;
   probe.adjoint = false;
   probe.g = g;
-  const bool brick = diffusion && g.ndim == 3 && aligned16(u0) && brick_adjoint_supported(probe) && strip_choice(probe, &sc);
+  const bool brick = diffusion && g.ndim == 3 && aligned16(u0) && brick_adjoint_supported(probe) && strip_choice(probe, &sc) &&
+                     brick_adjoint_faster(probe, tma);
   // A gradient written over lambda_T (lope_vjp in place): with two steps in all, a
   // pass of two would write cells of lambda_T that other blocks still read.
   const size_t bytes = size_t(npts(g)) * esize(g.dtype);

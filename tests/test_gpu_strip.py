@@ -408,8 +408,8 @@ def _dc(lope, g, st, u, lam, T, bcs):
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("shape,bcs", [((37, 380, 300), [1, 0, 1]), ((37, 380, 300), [0, 1, 0]),
-                                       ((130, 189, 204), [0, 0, 1]), ((130, 189, 204), [1, 1, 0])],
-                         ids=str)
+                                       ((130, 189, 204), [0, 0, 1]), ((130, 189, 204), [1, 1, 0]),
+                                       ((126, 200, 300), [1, 1, 1])], ids=str)
 @pytest.mark.parametrize("T,ckpt", [(13, 7), (4, 4)])
 def test_brick_adjoint_counts_every_cell_once(lope, dtype, shape, bcs, T, ckpt):
     """dL/dc on extents that are no multiple of a block's, sides of both kinds:
@@ -505,3 +505,23 @@ def test_depth_of_radius_two_batches(lope, kinds, passes):
     assert lope.launch_count() - n == passes + 1
     for g, u, o in zip(grids, ins, outs):
         assert torch.equal(_run(lope, g, st, u, 9, lope.Launch(DIRECT, 0, 0, 0, -1)), o)
+
+
+@pytest.mark.parametrize("dtype,shape,bcs,pairs", [
+    ("f32", (65, 256, 256), [1, 1, 1], False), ("f32", (65, 256, 256), [1, 0, 1], True),
+    ("f32", (65, 256, 256), [0, 0, 0], True), ("f32", (128, 200, 300), [1, 1, 1], True),
+    ("bf16", (128, 256, 256), [1, 1, 1], False), ("bf16", (128, 256, 256), [1, 0, 1], True),
+    ("bf16", (65, 256, 256), [1, 0, 1], False), ("bf16", (40, 600, 600), [1, 1, 1], True)], ids=str)
+def test_route_of_the_adjoint(lope, dtype, shape, bcs, pairs):
+    """Four steps back from one checkpoint: in pairs (zeroing, states 2 + 1, two passes,
+    the final sum) or one at a time (zeroing, 3 states, 4 steps, the final sum),
+    whichever is faster there."""
+    st = lope.Stencil.builtin("diff7", 0.1)
+    g = lope.Grid(shape, dtype, halo=1).set_boundaries(bcs)
+    u, _ = to_device(LI.uniform_field(1900, shape), dtype)
+    gT, _ = to_device(LI.normal_field(1901, shape), dtype)
+    _, ws = lope.forward_ckpt(g, st, u, 4, 4)
+    n = lope.launch_count()
+    grad, _ = lope.vjp(g, st, u, gT, 4, 4, reuse=True, workspace=ws)
+    assert lope.launch_count() - n == (6 if pairs else 9)
+    assert torch.equal(grad, _run(lope, g, st, gT, 4, lope.Launch(DIRECT, 0, 0, 0, -1)))
