@@ -323,8 +323,9 @@ bool strip_choice(StepArgs a, Choice* c) {
 // with the least estimated time per sweep.  A launch lasts as long as its busiest
 // SM, which the FP64 pipe binds: in us, 2.38 + 0.64 per sweep + 0.0467 (5 terms;
 // 0.091 with 9) per window row of 32 points that the SM computes.  Fitted to 71
-// timings on GB300 (within 20 %; at each of the 14 grids the fastest tile and depth
-// of those timed is the one estimated so).  us for 40 sweeps, 64 x 16 at depth 4
+// timings on GB300 (within 20 %), so another tile than 64 x 16 at depth 4 has to be
+// 8 % better by it (jacobi5 426 x 640 and a 3 x 3 table 362^2, 6 % better by the
+// estimate, took 80 -> 86 us for 12 sweeps).  us for 40 sweeps, 64 x 16 at depth 4
 // (the choice of shorter calls) against the estimate's: jacobi5 256^2 162 -> 111
 // (64 x 8, depth 4: 128 blocks instead of 64 for 152 SMs), 100 x 300 164 -> 84 (32 x 8,
 // depth 4), 512^2 252 -> 224, star9r2 700 x 900 1190 -> 602 (32 x 8, depth 1).
@@ -348,7 +349,8 @@ bool f64_choice(StepArgs a, Choice* c) {
           rows += int64_t((tx + 2 * R * (k - s) + 31) / 32) * (ty + 2 * R * (k - s));
         const int64_t blocks = ((g.n[2] + tx - 1) / tx) * ((g.n[1] + ty - 1) / ty);
         rows *= (blocks + kSms - 1) / kSms;
-        const double t = (2.38 + 0.64 * k + (0.0111 * terms - 0.0088) * double(rows)) / k;
+        double t = (2.38 + 0.64 * k + (0.0111 * terms - 0.0088) * double(rows)) / k;
+        if (tx == 64 && ty == 16 && k == 4) t /= 1.08;
         if (t < best) {
           best = t;
           *c = {kPathTrap, tx, ty, k};

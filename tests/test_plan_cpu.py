@@ -16,8 +16,8 @@ for (int f = 0; f < NF; ++f)
 """
 
 
-def _plan(L, shape, dtype, fn, bc, steps=12, scheme="euler"):
-    """(path, depth) of a call with aligned pointers."""
+def _plan(L, shape, dtype, fn, bc, steps=12, scheme="euler", tile=False):
+    """(path, depth) of a call with aligned pointers; tile: (path, tile, depth)."""
     if fn == "box2":
         w = np.arange(1.0, 26.0).reshape(5, 5) / 325.0
         st, halo, nf = L.Stencil.linear(w), 2, 1
@@ -34,6 +34,8 @@ def _plan(L, shape, dtype, fn, bc, steps=12, scheme="euler"):
     base = 1 << 44
     at = lambda k: [base + (k * nf + f) * 2 * field for f in range(nf)]  # noqa: E731
     plan, _ = L.lope_plan(g.handle, st.handle, at(0), at(1), at(2), steps, None)
+    if tile:
+        return plan.path, plan.tile_x, plan.tile_y, plan.tsteps
     return plan.path, plan.tsteps
 
 
@@ -87,6 +89,16 @@ def test_bricks_on_thin_grids(lope, dtype, shape, bc, want):
     """Thin grids whose blocks leave half of the SMs idle keep two sweeps per launch
     where those run (x and y sides Dirichlet)."""
     assert _plan(lope, shape, dtype, "diff7", bc) == want
+
+
+@pytest.mark.parametrize("fn,shape,want", [
+    ("jacobi5", (256, 256), (64, 8, 4)), ("jacobi5", (100, 300), (32, 8, 4)),
+    ("jacobi5", (426, 640), (64, 16, 4)), ("jacobi5", (511, 513), (64, 16, 4)),
+    ("jacobi5", (512, 512), (32, 8, 1)), ("star9r2", (700, 900), (32, 8, 1)),
+], ids=str)
+def test_tile_of_double_grids(lope, fn, shape, want):
+    """Another tile than 64 x 16 at depth 4 only where the estimate is clearly better."""
+    assert _plan(lope, shape, "f64", fn, [D, P], tile=True) == (TRAP,) + want
 
 
 @pytest.mark.parametrize("fn,dtype,shape,bc,scheme,path", [
