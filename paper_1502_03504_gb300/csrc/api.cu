@@ -252,10 +252,11 @@ int strip_depth(const StepArgs& a) {
   one.ksteps = 1;
   const bool tma = tma_supported(one);
   if (s.stages >= 2) {
-    // BF16 radius-2 tables (RK3 1000^2 Dirichlet 169 / 294, 4096^2 periodic 1475 / 1654;
-    // RK2 periodic 934 / 840) and the nonlinear shallow water with masks (RK3 BF16
-    // 848^2 Dirichlet 186 / 241, FP32 1000^2 243 / 255).
-    if (box2 && !f32) return side ? n < (1 << 17) : s.stages == 2 || n < (1 << 19);
+    // BF16 radius-2 tables (RK3 605 x 144 with y sides Dirichlet, 13 steps, 154 / 189,
+    // 1000^2 Dirichlet 169 / 294, 4096^2 periodic 1475 / 1654; RK2 periodic 934 / 840)
+    // and the nonlinear shallow water with masks (RK3 BF16 848^2 Dirichlet 186 / 241,
+    // FP32 1000^2 243 / 255).
+    if (box2 && !f32) return s.stages == 2 ? !side || n < (1 << 17) : !side && n < (1 << 19);
     return !(s.kind == kSweFlux && s.stages == 3 && side_x && tma && n >= (1 << 19) && n < (1 << 21));
   }
   // The state is past the trapezoid's 8 MB and short of the two-sweep tiles' 2^22 points:

@@ -105,6 +105,8 @@ def test_tile_of_double_grids(lope, fn, shape, want):
     ("box2", "bf16", (1000, 1000), [D, D], "rk2", TMA),
     ("box2", "bf16", (1000, 1000), [P, P], "rk2", STRIP),
     ("box2", "bf16", (1000, 1000), [P, P], "rk3", TMA),
+    ("box2", "bf16", (144, 600), [D, P], "rk3", TMA),
+    ("box2", "bf16", (144, 600), [D, P], "rk2", STRIP),
     ("box2", "f32", (1000, 1000), [D, D], "rk3", STRIP),
     ("swe_flux", "f32", (848, 848), [D, D], "rk3", TMA),
     ("swe_flux", "f32", (848, 848), [P, P], "rk3", STRIP),
