@@ -661,8 +661,9 @@ def form_swe_flux(L, LI, torch, dev, peak):
 
 def form_rk3(L, LI, torch, dev, peak):
     """SSP-RK3 steps of the nonlinear shallow water, 4096^2 x 3 FP32, 50 steps:
-    fused trapezoid steps (stage states in shared memory) against one launch
-    per stage (TMA tiles, stage states in HBM) and against 150 plain sweeps."""
+    the plan a call takes (register strips: a step's stages as levels), fused
+    trapezoid steps (stage states in shared memory), one launch per stage (TMA
+    tiles, stage states in HBM) and 150 plain sweeps."""
     n, T = 4096, 50
     f = _flux_fields(LI, torch, dev, n, "f32", 1105)
     o = [torch.empty_like(x) for x in f]
@@ -682,10 +683,15 @@ def form_rk3(L, LI, torch, dev, peak):
     ms_fused, tx, ty, k = best
     ms_stage = _time(torch, lambda: L.apply(g, s, f, out=o, work=w, nsteps=T,
                                             launch=L.Launch(1, 0, 0, 0, -1)), reps=3)
+    ms_plan = _time(torch, lambda: L.apply(g, s, f, out=o, work=w, nsteps=T), reps=3)
+    plan = L.plan(g, s, f, o, w, nsteps=T)[0]
     e = L.Stencil.builtin("swe_flux", 0.02, 1.0, 0.5, 1.0)
     ms_euler = _time(torch, lambda: L.apply(g, e, f, out=o, work=[x[0] for x in w], nsteps=3 * T), reps=3)
     pts = n * n * T
     return {"workload": "SSP-RK3 nonlinear shallow water 4096^2 x3 FP32 periodic x50 steps (150 stages)",
+            "ms": ms_plan, "path": plan.path, "rk_steps_per_s": pts / (ms_plan / 1e3),
+            "alg_GBps": 24 * pts / (ms_plan / 1e3) / 1e9,
+            "frac_of_peak": 24 * pts / (ms_plan / 1e3) / 1e9 / peak,
             "fused_trapezoid_ms": ms_fused, "fused_choice": {"tile": [tx, ty], "tsteps": k},
             "fused_rk_steps_per_s": pts / (ms_fused / 1e3),
             "fused_alg_GBps": 24 * pts / (ms_fused / 1e3) / 1e9,

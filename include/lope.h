@@ -220,8 +220,17 @@ lope_status lope_apply_host(const lope_grid* grid, const lope_stencil* stencil,
  *              radius-1 star), 6 (three-field star) or 4, or less: 4, 2, 1;
  *              a sweep count that is no multiple ends with launches of 4, 2
  *              and 1 sweeps.  Multi-stage steps run one step per launch.
- *              The planner's choice for calls of 12 or more sweeps; shorter
- *              calls take the paths below.
+ *              3D: register bricks, blocks of 64 x 64 columns that march along
+ *              z.  diff7 and radius-1 star weight tables, plain sweeps, FP32 rows
+ *              of any pitch, BF16 rows of a multiple of 4; at least 64 points
+ *              along x and y.  tsteps is 4 or 2; what an odd count leaves over
+ *              runs one sweep on the path of short calls.
+ *              The planner's choice for calls of 12 or more sweeps, in 3D on rows
+ *              TMA cannot stage and else from 2^22 points on; shorter calls take
+ *              the paths below.  So do functions that measured faster there:
+ *              radius-2 box tables with Dirichlet sides and functions of several
+ *              fields with Dirichlet x sides on states that stay in L2, and thin
+ *              3D grids; some radius-2 functions run at depth 2.
  *            For grids whose row pitch is not a multiple of 16 bytes the
  *            planner takes trapezoid tiles fusing 4 sweeps in 2D (128 x 32
  *            for one field, 64 x 16 for several) and the plane march in 3D.

@@ -233,7 +233,8 @@ constexpr int kSms = 152;  // of a GB300: plans are made without a CUDA call
 
 // The register strips serve calls of at least kStripSteps sweeps (or steps).
 // Shorter calls keep the plans documented for them (see lope.h): callers that
-// query or log the plan of a short call see the path they always saw.
+// query or log the plan of a short call see the path they always saw.  The limit is
+// that, not a measured one.
 constexpr int64_t kStripSteps = 12;
 
 // Depth of a 2D call in strips, or 0 where the plan of shorter calls is as fast.  The
@@ -379,7 +380,7 @@ Choice default_choice(const Geom& g, const StencilDesc& s, const void* const* in
     // 8192^2 x50 3.03 -> 1.72 ms; linear shallow water 4096^2 x3 x200 FP32 7.86
     // -> 2.60 ms, BF16 7.17 -> 2.40; RK3 nonlinear shallow water FP32 4096^2 x50
     // steps 14.2 -> 5.15 ms; a run-time compiled Gray-Scott FP32 4096^2 x100
-    // 3.99 -> 1.46 ms.  FP64 is bound by its arithmetic and keeps to trapezoid
+    // 3.99 -> 1.49 ms.  FP64 is bound by its arithmetic and keeps to trapezoid
     // tiles (256^2 x100: 0.28 ms, 0.46 in strips).
     StepArgs b = a;
     if (in)
@@ -807,8 +808,10 @@ lope_status forward_ckpt_impl(const lope_grid* grid, const lope_stencil* st, con
                               cudaStream_t stream) {
   void* tmp = ws + L.off_tmp;
   const void* cur = u0;
-  // A segment's sweeps take the strips / bricks from half their planner's count
-  // on: the segments follow one another, so their fill is paid once per depth.
+  // Segments of 6 sweeps or more take the strips / bricks where longer calls do
+  // (whole calls with segments of 6 to 12 sweeps, against the plans of short ones:
+  // jacobi5 100 x 200 1.12, 2048^2 FP32 1.08 and BF16 1.33 times as fast, star9r2
+  // 1000^2 1.23, 2048^2 1.03).
   StepArgs probe = base_args(grid->g, st->s, nullptr, nullptr);
   probe.in[0] = u0;
   Choice sc;

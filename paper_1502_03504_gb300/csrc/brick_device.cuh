@@ -25,15 +25,18 @@
 // own over the first and last steps.  Each level is rounded to the storage
 // precision: bitwise the result of K one-sweep launches.
 //
-// What bounds it: instruction issue and its latencies, with 8 warps per SM.
+// What bounds it: latency, with 8 warps per SM: issue is busy 65 % of the time at
+// 512^3, and a warp waits on exchange rows and planes in shared memory (0.53 per
+// issue) and on staged planes (0.29), hardly on the barrier (0.06).
 // One block of 16 half-warps x 4 rows and up to 255 registers measured best
 // (diff7 FP32, us per sweep, 512^3 Dirichlet / 256^3 periodic / 130 x 500 x 510):
 //   K = 4: 73.5 / 13.4 / 33.9 (244 registers)
 //   K = 3: 77.2 / 15.1 / 37.3 (197); 12 half-warps, two blocks of 168: 95 / 18 / 51
 //   K = 2: 95.5 / 17.5 / 52; 5 or 6 rows per thread were no better
-// against 109 (two sweeps per launch) / 25.4 / 75.7 (one) on the z-marches.  Tiles
-// 64 columns wide waste less of a 256- or 512-wide grid than 128 (a warp per
-// row): 1.97 -> 1.41 times the points at 256^3.
+// against 109 (two sweeps per launch) / 25.4 / 75.7 (one) on the z-marches.  The
+// blocks cover 1.56 times the points of a periodic 256^3 grid (five blocks of 64 along
+// x and y) and 1.27 times those of a Dirichlet 512^3; 128 columns (a warp per row)
+// would cover 1.88 times the former.
 #pragma once
 
 #include "strip_device.cuh"

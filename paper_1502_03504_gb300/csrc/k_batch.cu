@@ -129,7 +129,9 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(Op op, BatchPlanDe
 // kept about 45 registers of its loop alive across the march and spilled it
 // (512 grids of sides 64..2048, jacobi5 x20, 5.9e8 points: 9.5 ms, with all
 // depths in one kernel 11.6 ms; this form 5.09 ms, the two-sweep shared-memory
-// tiles it replaced 12.5 ms).  A batch with Dirichlet sides mixes masked and
+// tiles it replaced 12.5 ms).  One kernel holds the marches of aligned and of other
+// rows, masked and plain, and at depth 8 still spills some (jacobi5 a 104-byte frame,
+// 40 without masks).  A batch with Dirichlet sides mixes masked and
 // plain units on an SM: at radius 1 all of them then run on packed pairs, whose
 // code is smaller (5.60 ms on scalars, 5.40 with pairs in the masked units only);
 // at radius 2 only the masked ones (256 odd grids x16 at depth 4: 3.93 ms, 4.05 on

@@ -446,8 +446,8 @@ struct Strip {
 // The cut of one grid into units.  Inner strips are cut into nc chunks, strips
 // that touch a Dirichlet x side into nce >= nc shorter ones (their masks cost
 // about half as much again per row, and with all units resident at once the
-// slowest sets the time); the first and last chunk of a grid with Dirichlet y
-// sides are shortened the same way (ychunk).  Units of edge strips come first.
+// slowest sets the time); the first chunk of a grid whose low y side is Dirichlet
+// is shortened the same way (top).  Units of edge strips come first.
 struct StripCut {
   int strips;      // all strips
   int el, er;      // 1: the first / last strip is cut into nce chunks

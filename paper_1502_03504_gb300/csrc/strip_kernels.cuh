@@ -1,6 +1,6 @@
 // Host-side runner of the register strips (strip_device.cuh): depths and block
 // shape per function shape, the cut of the grid into strips and chunks, and
-// the launch.  Shared by k_strip.cu (builtins) and jit.cu (run-time compiled
+// the launch.  Shared by k_strip_*.cu (builtins) and jit.cu (run-time compiled
 // local functions).
 #pragma once
 
@@ -20,8 +20,9 @@ namespace {
 // 8192^2, per sweep: 25 us at depth 4, 18.5 at 6, 17.2 at 8); three-field star
 // functions: 6 (linear shallow water FP32 4096^2: 19.0 us at 4, 12.9 at 6);
 // radius 2 and box functions: 4 (star9r2 FP32 8192^2: 33.9 us at 4, 41 at
-// 6, where it spills; nonlinear shallow water 30.8 and 41).  What is left of the
-// sweep count runs at depths 4, 2 and 1.
+// 6, where it spills; nonlinear shallow water 30.8 and 41).  Radius-2 box tables and
+// run-time compiled radius-2 functions of three fields spill at 4 already and run at 2
+// by default (api.cu, strip_depth).  What is left of the sweep count runs at depths 4, 2 and 1.
 constexpr int strip_kmax(int nf, int radius, bool star) {
   if (radius > 1 || !star) return 4;
   return nf == 1 ? 8 : nf == 3 ? 6 : 4;
@@ -42,7 +43,8 @@ template <class T, int R, int NF, int K, int STG> struct StripCfg {
   // 24 sweeps: linear shallow water 319 -> 290 us, nonlinear 804 -> 777, with
   // Dirichlet sides 1306 -> 998), FP32 only with masks (nonlinear shallow water
   // with Dirichlet sides 1171 -> 1073 us, star9r2 298 -> 278; without masks
-  // star9r2 8192^2 x50 1.70 -> 1.97 ms).  Element copies at depth 8 would spill.
+  // star9r2 8192^2 x50 1.70 -> 1.97 ms).  Element copies at depth 8 spill
+  // on scalars already (with masks a 72-byte frame) and stay on them.
   static constexpr int pm(bool vec, bool dirichlet) {
     return sizeof(T) == 2 ? 2 : !dirichlet || (!vec && K == 8) ? 0 : 1;
   }
